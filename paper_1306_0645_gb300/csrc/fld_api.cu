@@ -1338,8 +1338,8 @@ fld_status assemble_coarse(fld_ctx* c) {
     { const double nc = (double)Lc.d.n;
       KScope k(c, K_COARSE_SETUP, 16.0 * nc * nc);
       // the mixed solver's cycle is FP32 throughout, also on a one-level grid
-      if (c->mixed) launch_coarse_setup<float>(Lc.d, Lc.A32, c->dense, c->ainv, c->sc, true, s);
-      else launch_coarse_setup<double>(Lc.d, Lc.A64, c->dense, c->ainv, c->sc, false, s); }
+      if (c->mixed) launch_coarse_setup<float>(Lc.d, Lc.A32, c->dense, c->ainv, c->sc, c->counter + 48, true, s);
+      else launch_coarse_setup<double>(Lc.d, Lc.A64, c->dense, c->ainv, c->sc, c->counter + 48, false, s); }
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaMemcpyAsync(c->h_sc, c->sc, NUM_SLOTS * sizeof(double), cudaMemcpyDeviceToHost, s));
     return FLD_OK;

@@ -1,7 +1,7 @@
 // k_mg.cu -- geometric multigrid V-cycle pieces for the 7-point FLD system
 // (the preconditioner of Table 1): coarse operators, red/black Gauss-Seidel
-// and weighted Jacobi smoothing, residual, full-weighting restriction,
-// trilinear prolongation, and the dense coarsest-grid solve.
+// and weighted Jacobi smoothing, residual, full-weighting restriction and
+// trilinear prolongation (the dense coarsest-grid solve: k_coarse.cu).
 //
 // Cell-centred full coarsening; operators by rediscretisation (coarse face
 // weight = sum of the 4 fine face weights across the coarse face / 16,
@@ -276,200 +276,6 @@ __global__ void k_prolong_add(Dims f, Dims cd, const T* __restrict__ ec, T* __re
     }
 }
 
-// ---------------------------------------------------------- coarsest grid
-
-template <class T>
-__global__ void k_dense_build(Dims d, Op<T> A, double* __restrict__ M) {
-    const long long n = d.n;
-    GRID_LOOP(c, n) {
-        double* row = M + c * n;
-        for (long long q = 0; q < n; q++) row[q] = 0.0;
-    }
-    // rows are owned by one thread each, so the adds below do not race
-    GRID_LOOP(c, n) {
-        int i, j, k;
-        cell_ijk(c, d, i, j, k);
-        double* row = M + c * n;
-        const long long sy = d.nx, sz = (long long)d.nx * d.ny;
-        double diag = (double)A.m[c];
-        auto add = [&](T wt, long long nb) {
-            const double w = (double)wt;
-            diag += w;
-            row[nb] -= w;
-        };
-        if (i > 0) add(A.wx[c], c - 1); else if (d.px) add(A.wx[c], c + d.nx - 1);
-        if (i < d.nx - 1) add(A.wx[c + 1], c + 1); else if (d.px) add(A.wx[c - (d.nx - 1)], c - (d.nx - 1));
-        if (j > 0) add(A.wy[c], c - sy); else if (d.py) add(A.wy[c], c + (long long)(d.ny - 1) * sy);
-        if (j < d.ny - 1) add(A.wy[c + sy], c + sy); else if (d.py) add(A.wy[c - (long long)(d.ny - 1) * sy], c - (long long)(d.ny - 1) * sy);
-        if (k > 0) add(A.wz[c], c - sz); else if (d.pz) add(A.wz[c], c + (long long)(d.nz - 1) * sz);
-        if (k < d.nz - 1) add(A.wz[c + sz], c + sz); else if (d.pz) add(A.wz[c - (long long)(d.nz - 1) * sz], c - (long long)(d.nz - 1) * sz);
-        row[c] += diag;
-    }
-}
-
-// One CTA: in-place Cholesky of the dense SPD matrix M (row-major, lower
-// triangle becomes L), then the explicit inverse Ainv = L^-T L^-1, one
-// column per thread.  A non-positive pivot sets sc[S_BAD] = 2.
-__global__ void k_chol_inverse(int n, double* M, double* Ainv, double* sc) {
-    __shared__ int fail;
-    if (threadIdx.x == 0) fail = 0;
-    __syncthreads();
-    for (int j = 0; j < n; j++) {
-        if (threadIdx.x == 0) {
-            const double piv = M[(long long)j * n + j];
-            if (!(piv > 0.0)) { fail = 1; M[(long long)j * n + j] = 1.0; }
-            else M[(long long)j * n + j] = sqrt(piv);
-        }
-        __syncthreads();
-        const double ljj = M[(long long)j * n + j];
-        for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x) M[(long long)i * n + j] /= ljj;
-        __syncthreads();
-        // trailing update of the lower triangle: M[i][k] -= L[i][j] L[k][j], j < k <= i
-        for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x) {
-            const double lij = M[(long long)i * n + j];
-            for (int k = j + 1; k <= i; k++) M[(long long)i * n + k] -= lij * M[(long long)k * n + j];
-        }
-        __syncthreads();
-    }
-    if (fail && threadIdx.x == 0) sc[S_BAD] = 2.0;
-    // inverse, column t: L y = e_t, then L^T x = y, written in Ainv[:, t]
-    for (int t = threadIdx.x; t < n; t += blockDim.x) {
-        for (int i = 0; i < t; i++) Ainv[(long long)i * n + t] = 0.0;
-        for (int i = t; i < n; i++) {
-            double s = (i == t) ? 1.0 : 0.0;
-            for (int k = t; k < i; k++) s -= M[(long long)i * n + k] * Ainv[(long long)k * n + t];
-            Ainv[(long long)i * n + t] = s / M[(long long)i * n + i];
-        }
-        for (int i = n - 1; i >= 0; i--) {
-            double s = Ainv[(long long)i * n + t];
-            for (int k = i + 1; k < n; k++) s -= M[(long long)k * n + i] * Ainv[(long long)k * n + t];
-            Ainv[(long long)i * n + t] = s / M[(long long)i * n + i];
-        }
-    }
-}
-
-// Coarsest-grid setup for small grids, one CTA with the matrix in shared
-// memory: Cholesky M = L L^T in precision T (the trailing update spread over
-// all threads), X = L^-1 by forward substitution (one column per thread),
-// and the inverse Ainv = X^T X, written as FP64 (exactly symmetric).  The
-// mixed-precision solver takes T = float: its whole V-cycle is FP32.  A
-// non-positive pivot sets sc[S_BAD] = 2.
-template <class T>
-__global__ void __launch_bounds__(1024) k_chol_inverse_smem(int n, const double* __restrict__ M,
-                                                            double* __restrict__ Ainv, double* sc) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* L = reinterpret_cast<T*>(smem_raw);   // n x n, row-major
-    T* X = L + (long long)n * n;             // n x n, row-major, lower triangle
-    __shared__ int fail;
-    const int tid = threadIdx.x, nt = blockDim.x;
-    if (tid == 0) fail = 0;
-    for (int q = tid; q < n * n; q += nt) {
-        L[q] = (T)M[q];
-        X[q] = T(0);
-    }
-    __syncthreads();
-    for (int j = 0; j < n; j++) {
-        if (tid == 0) {
-            const T piv = L[j * n + j];
-            if (!(piv > T(0))) { fail = 1; L[j * n + j] = T(1); }
-            else L[j * n + j] = sqrt(piv);
-        }
-        __syncthreads();
-        const T ljj = L[j * n + j];
-        for (int i = j + 1 + tid; i < n; i += nt) L[i * n + j] /= ljj;
-        __syncthreads();
-        // trailing update of the lower triangle: (i, k) with j < k <= i
-        const int m = n - j - 1;
-        for (int q = tid; q < m * m; q += nt) {
-            const int i = j + 1 + q / m, k = j + 1 + q % m;
-            if (k <= i) L[i * n + k] -= L[i * n + j] * L[k * n + j];
-        }
-        __syncthreads();
-    }
-    for (int t = tid; t < n; t += nt)
-        for (int i = t; i < n; i++) {
-            T v = (i == t) ? T(1) : T(0);
-            for (int k = t; k < i; k++) v -= L[i * n + k] * X[k * n + t];
-            X[i * n + t] = v / L[i * n + i];
-        }
-    __syncthreads();
-    for (int q = tid; q < n * n; q += nt) {
-        const int a = q / n, b = q - a * n;
-        T v = T(0);
-        for (int i = a > b ? a : b; i < n; i++) v += X[i * n + a] * X[i * n + b];
-        Ainv[q] = (double)v;
-    }
-    if (fail && tid == 0) sc[S_BAD] = 2.0;
-}
-
-// Coarsest-grid inverse for n <= 128, one CTA of 32 x 32 threads with the
-// matrix in shared memory: in-place Gauss-Jordan elimination without
-// pivoting (stable for the symmetric positive definite operator).  Step k
-// replaces the matrix M by
-//   M'[k][k] = 1/p,  M'[k][j] = M[k][j]/p,  M'[i][k] = -M[i][k]/p,
-//   M'[i][j] = M[i][j] - M[i][k] M[k][j]/p      (p = M[k][k] > 0),
-// every entry at once (read phase, barrier, write phase); after n steps M
-// holds the inverse.  Each thread owns the entries (ty + 32 a, tx + 32 b).
-// The result is written as FP64.  A non-positive pivot sets sc[S_BAD] = 2.
-constexpr int GJ_MAX = 128;
-template <class T, int PT>   // PT = entries per thread and axis, n <= 32 PT
-__global__ void __launch_bounds__(1024) k_gj_inverse_smem(int n, const double* __restrict__ M,
-                                                          double* __restrict__ Ainv, double* sc) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* A = reinterpret_cast<T*>(smem_raw);
-    __shared__ int fail;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    if (threadIdx.x == 0) fail = 0;
-    for (int q = threadIdx.x; q < n * n; q += 1024) A[q] = (T)M[q];
-    __syncthreads();
-    for (int k = 0; k < n; k++) {
-        T p = A[k * n + k];
-        if (!(p > T(0))) {
-            if (threadIdx.x == 0) fail = 1;
-            p = T(1);
-        }
-        const T ip = T(1) / p;
-        T nv[PT][PT];
-#pragma unroll
-        for (int a = 0; a < PT; a++) {
-            const int i = ty + 32 * a;
-#pragma unroll
-            for (int b = 0; b < PT; b++) {
-                const int j = tx + 32 * b;
-                if (i < n && j < n) {
-                    if (i == k && j == k) nv[a][b] = ip;
-                    else if (i == k) nv[a][b] = A[k * n + j] * ip;
-                    else if (j == k) nv[a][b] = -A[i * n + k] * ip;
-                    else nv[a][b] = A[i * n + j] - A[i * n + k] * (A[k * n + j] * ip);
-                }
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int a = 0; a < PT; a++) {
-            const int i = ty + 32 * a;
-#pragma unroll
-            for (int b = 0; b < PT; b++) {
-                const int j = tx + 32 * b;
-                if (i < n && j < n) A[i * n + j] = nv[a][b];
-            }
-        }
-        __syncthreads();
-    }
-    for (int q = threadIdx.x; q < n * n; q += 1024) Ainv[q] = (double)A[q];
-    if (fail && threadIdx.x == 0) sc[S_BAD] = 2.0;
-}
-
-template <class T>
-__global__ void k_coarse_apply(int n, const double* __restrict__ Ainv, const T* __restrict__ r,
-                               T* __restrict__ z) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int j = 0; j < n; j++) s += Ainv[(long long)j * n + i] * (double)r[j];
-        z[i] = (T)s;
-    }
-}
-
 // ---------------------------------------------------------------- launchers
 
 static const int TPB = 256;
@@ -521,66 +327,17 @@ void launch_prolong_add(const Dims& f, const Dims& c, const T* ec, T* zf, cudaSt
     ColShape sh = col_shape(f);
     k_prolong_add<T><<<sh.grid, sh.block, 0, s>>>(f, c, ec, zf);
 }
-// shared memory of the in-CTA setup for an n x n matrix in precision T
-// (factor and inverse), and whether it fits
-static size_t chol_smem_bytes(long long n, size_t ts) { return 2 * (size_t)n * (size_t)n * ts; }
-static const size_t CHOL_SMEM_MAX = 200 * 1024;
-
-template <class T>
-void launch_coarse_setup(const Dims& d, Op<T> A, double* dense, double* ainv, double* sc, bool fp32,
-                         cudaStream_t s) {
-    k_dense_build<T><<<1, TPB, 0, s>>>(d, A, dense);
-    const size_t ts = fp32 ? sizeof(float) : sizeof(double);
-    if (d.n <= GJ_MAX) {
-        const size_t gb = (size_t)d.n * (size_t)d.n * ts;
-        const int n = (int)d.n;
-        auto go = [&](auto kern) {
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gb);
-            kern<<<1, 1024, gb, s>>>(n, dense, ainv, sc);
-        };
-        if (fp32) {
-            if (n <= 32) go(k_gj_inverse_smem<float, 1>);
-            else if (n <= 64) go(k_gj_inverse_smem<float, 2>);
-            else go(k_gj_inverse_smem<float, 4>);
-        } else {
-            if (n <= 32) go(k_gj_inverse_smem<double, 1>);
-            else if (n <= 64) go(k_gj_inverse_smem<double, 2>);
-            else go(k_gj_inverse_smem<double, 4>);
-        }
-        return;
-    }
-    const size_t bytes = chol_smem_bytes(d.n, ts);
-    if (bytes <= CHOL_SMEM_MAX) {
-        if (fp32) {
-            cudaFuncSetAttribute(k_chol_inverse_smem<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-            k_chol_inverse_smem<float><<<1, 1024, bytes, s>>>((int)d.n, dense, ainv, sc);
-        } else {
-            cudaFuncSetAttribute(k_chol_inverse_smem<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-            k_chol_inverse_smem<double><<<1, 1024, bytes, s>>>((int)d.n, dense, ainv, sc);
-        }
-        return;
-    }
-    const int threads = d.n < 1024 ? (int)((d.n + 31) / 32 * 32) : 1024;
-    k_chol_inverse<<<1, threads, 0, s>>>((int)d.n, dense, ainv, sc);
-}
-template <class T>
-void launch_coarse_apply(int n, const double* ainv, const T* r, T* z, cudaStream_t s) {
-    k_coarse_apply<T><<<(n + 127) / 128, 128, 0, s>>>(n, ainv, r, z);
-}
-
 #define INST(T)                                                                                    \
     template void launch_invd<T>(const Dims&, Op<T>, const Op<T>&, cudaStream_t);                   \
     template void launch_coarsen<T>(const Dims&, const Dims&, Op<T>, Op<T>, cudaStream_t);           \
     template void launch_coarsen_bnd<T>(const Dims&, const Dims&, int, Bnd, Bnd, Op<T>, cudaStream_t); \
-    template void launch_coarse_setup<T>(const Dims&, Op<T>, double*, double*, double*, bool, cudaStream_t); \
     template void launch_smooth_zero<T>(const Dims&, Op<T>, const T*, T*, cudaStream_t);            \
     template void launch_rb_colour<T>(const Dims&, Op<T>, const T*, T*, int, cudaStream_t);         \
     template void launch_jacobi<T>(const Dims&, Op<T>, const T*, const T*, T*, double, bool,        \
                                    cudaStream_t);                                                  \
     template void launch_residual<T>(const Dims&, Op<T>, const T*, const T*, T*, cudaStream_t);     \
     template void launch_restrict<T>(const Dims&, const Dims&, const T*, T*, cudaStream_t);         \
-    template void launch_prolong_add<T>(const Dims&, const Dims&, const T*, T*, cudaStream_t);      \
-    template void launch_coarse_apply<T>(int, const double*, const T*, T*, cudaStream_t);
+    template void launch_prolong_add<T>(const Dims&, const Dims&, const T*, T*, cudaStream_t);
 INST(float)
 INST(double)
 

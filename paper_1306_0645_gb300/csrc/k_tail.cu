@@ -316,13 +316,19 @@ __device__ void tail_up(const TailLevel<T>& L, Vec<T> v, const Dims& cd, const T
         }
 }
 
-// z = A^-1 r on the coarsest grid with the stored explicit inverse.
+// z = A^-1 r on the coarsest grid with the stored explicit inverse: a warp
+// per row, the row's products summed by lanes.  (One thread per row summed n
+// FP64 products in a serial chain: 16 of them take 2 us on this GPU's FP64
+// pipe.)
 template <bool CG, class T, class Sync>
 __device__ void tail_coarsest(int n, const double* ainv, Vec<T> v, int tid, int nth, Sync sync) {
-    TAIL_LOOP(row, n) {
+    const int lane = threadIdx.x & 31;
+    for (int row = tid >> 5; row < n; row += nth >> 5) {
+        const double* a = ainv + (long long)row * n;
         double acc = 0.0;
-        for (int q = 0; q < n; q++) acc += ainv[q * n + row] * (double)ldw<CG>((const T*)v.r, q);
-        v.z[row] = (T)acc;
+        for (int q = lane; q < n; q += 32) acc += a[q] * (double)ldw<CG>((const T*)v.r, q);
+        acc = warp_sum(acc);
+        if (lane == 0) v.z[row] = (T)acc;
     }
     sync();
 }

@@ -188,10 +188,12 @@ template <class T>
 void launch_restrict(const Dims& f, const Dims& c, const T* rf, T* rc, cudaStream_t s);
 template <class T>
 void launch_prolong_add(const Dims& f, const Dims& c, const T* ec, T* zf, cudaStream_t s);
-// Coarsest grid: dense matrix, Cholesky, explicit inverse (one CTA; in
-// shared memory and in FP32 when fp32 and the matrix fits, else FP64).
+// ---- coarsest grid (k_coarse.cu): the explicit inverse in ainv (FP64, n x n;
+// fp32: of FP32 accuracy up to 160 cells, else FP64 accuracy).  dense: n x n
+// FP64 words of scratch; flag: one word of scratch; a non-positive pivot
+// sets sc[S_BAD] = 2.
 template <class T>
-void launch_coarse_setup(const Dims& d, Op<T> A, double* dense, double* ainv, double* sc, bool fp32,
+void launch_coarse_setup(const Dims& d, Op<T> A, double* dense, double* ainv, double* sc, unsigned* flag, bool fp32,
                          cudaStream_t s);
 template <class T>
 void launch_coarse_apply(int n, const double* ainv, const T* r, T* z, cudaStream_t s);
