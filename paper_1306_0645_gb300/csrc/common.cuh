@@ -251,8 +251,50 @@ struct DotAcc<float> {
         hi = t;
         lo = __fadd_rn(lo, __fadd_rn(err, e));
     }
+    // adds another pair; symmetric in the two, so lanes that merge each
+    // other's pairs hold the same sum
+    __device__ __forceinline__ void merge(const DotAcc& u) {
+        const float t = __fadd_rn(hi, u.hi);
+        const float bp = __fsub_rn(t, hi);
+        const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, bp)), __fsub_rn(u.hi, bp));
+        lo = __fadd_rn(__fadd_rn(lo, u.lo), err);
+        hi = t;
+    }
     __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
+
+// One row's part (every g-th entry from q0) of the coarsest inverse times r,
+// summed over g lanes.  FP32 solver: the inverse as a pair of floats, the
+// products split exactly and summed in a compensated pair on the FP32 pipe;
+// FP64 solver: FP64.
+template <int G, class T, class R>
+__device__ __forceinline__ T coarse_row(const double* ainv, int n, int row, int q0, R r) {
+    if constexpr (sizeof(T) == 4) {
+        const float2* a = reinterpret_cast<const float2*>(ainv) + (long long)row * n;
+        DotAcc<float> s;
+        for (int q = q0; q < n; q += G) {
+            const float2 v = a[q];
+            const float x = r(q);
+            s.add(v.x, x);
+            s.lo = fmaf(v.y, x, s.lo);
+        }
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) {
+            DotAcc<float> u;
+            u.hi = __shfl_xor_sync(0xffffffffu, s.hi, o);
+            u.lo = __shfl_xor_sync(0xffffffffu, s.lo, o);
+            s.merge(u);
+        }
+        return s.hi + s.lo;
+    } else {
+        const double* a = ainv + (long long)row * n;
+        double s = 0.0;
+        for (int q = q0; q < n; q += G) s = fma(a[q], r(q), s);
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        return s;
+    }
+}
 
 constexpr int FLAT_MAX_BLOCKS = 152 * 16;
 

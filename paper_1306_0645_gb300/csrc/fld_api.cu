@@ -545,15 +545,7 @@ void vcycle(fld_ctx* c, int l, const T* r, T* z, const RedArgs* dot = nullptr, b
             // smoothing, residual, transfers: about 30 words per cell
             bytes += 30.0 * (double)Q.d.n * ts;
         }
-        // the small levels in one CTA's shared memory, if their vectors fit
-        ta.small_from = ta.nlev;
-        for (int q = 0; q < ta.nlev; q++)
-            if (ta.L[q].d.n <= TAIL_SMALL_CELLS) {
-                size_t cells = 0;
-                for (int u = q; u < ta.nlev; u++) cells += (size_t)ta.L[u].d.n;
-                if (3 * cells * sizeof(T) <= TAIL_SMEM_MAX) ta.small_from = q;
-                break;
-            }
+        plan_tail<T>(ta, c->tail_cluster, false);
         KScope k(c, K_VTAIL, bytes);
         launch_vtail<T>(ta, c->tail_cluster, s);
         return;
@@ -960,7 +952,7 @@ fld_status ps_enqueue(std::vector<fld_ctx*> cs, cudaStream_t s) {
     size_t smem = 0;
     for (int i = 0; i < pb.n; i++) {
         pb.req[i] = cs[i]->ps_req;
-        const size_t b = psolve_smem_bytes(cs[i]->ps_host);
+        const size_t b = (size_t)cs[i]->ps_host.v.smem_bytes;
         if (b > smem) smem = b;
     }
     {
@@ -2116,16 +2108,9 @@ fld_status fld_create(fld_ctx** out, const fld_grid* g, const fld_params* p, voi
             t.z = (float*)(q == 0 ? c->cg[1] : Q.z);
             t.t = (float*)Q.t;
         }
-        ta.small_from = ta.nlev;
-        for (int q = 0; q < ta.nlev; q++)
-            if (ta.L[q].d.n <= TAIL_SMALL_CELLS) {
-                size_t cells = 0;
-                for (int u = q; u < ta.nlev; u++) cells += (size_t)ta.L[u].d.n;
-                if (3 * cells * sizeof(float) <= TAIL_SMEM_MAX) ta.small_from = q;
-                break;
-            }
         ta.ainv = c->ainv;   // filled by every assembly
-        R.cta = psolve_cta_bytes(ta) <= PS_SMEM_MAX ? 1 : 0;
+        R.cta = plan_tail<float>(ta, PS_CLUSTER, true) ? 1 : 0;
+        if (!R.cta) plan_tail<float>(ta, PS_CLUSTER, false);
         R.x = (float*)c->cg[5];
         R.p = (float*)c->cg[2];
         R.q = (float*)c->cg[4];

@@ -57,6 +57,21 @@ __device__ __forceinline__ void dense_row(const Dims& d, const Op<T>& A, int c, 
     row[c] = (M)diag;
 }
 
+// Entry i of the coarsest inverse as its solver reads it: FP64, or a float
+// pair high + low (FP32 solver).
+template <class T>
+__device__ __forceinline__ void put_inv(double* X, long long i, double v) {
+    if constexpr (sizeof(T) == 4) {
+        const float h = (float)v;
+        reinterpret_cast<float2*>(X)[i] = make_float2(h, (float)(v - (double)h));
+    } else {
+        X[i] = v;
+    }
+}
+// FP32 scratch copy of the inverse
+template <class T>
+__device__ __forceinline__ void put_inv(float* X, long long i, double v) { X[i] = (float)v; }
+
 // In-place inverse of the n x n matrix held by S x S threads, entry
 // (ty + S q, tx + S b) in a[q][b]; buf: 4 S PT values of shared memory.
 // Step k: p = M[k][k]; M'[k][k] = 1/p, M'[k][j] = M[k][j]/p,
@@ -143,7 +158,7 @@ __global__ void __launch_bounds__(S* S) k_gj_inverse(Dims d, Op<T> A, O* __restr
 #pragma unroll
         for (int b = 0; b < PT; b++) {
             const int i = ty + S * q, j = tx + S * b;
-            if (i < n && j < n) X[(long long)i * n + j] = (O)a[q][b];
+            if (i < n && j < n) put_inv<T>(X, (long long)i * n + j, (double)a[q][b]);
         }
     if (!ok && threadIdx.x == 0) {
         if (flag) *flag = 1u;
@@ -352,7 +367,7 @@ __global__ void __launch_bounds__(256) k_coarse_refine(Dims d, Op<T> A, const fl
     __syncthreads();
     for (int q = threadIdx.x; q < n * CB; q += 256) {
         const int c = c0 + q % CB;
-        if (c < n) X[(long long)(q / CB) * n + c] = x[q];
+        if (c < n) put_inv<T>(X, (long long)(q / CB) * n + c, x[q]);
     }
     if (!good && threadIdx.x == 0) *flag = 1u;
 }
@@ -403,6 +418,8 @@ __global__ void k_chol_inverse(Dims d, Op<T> A, double* M, double* Ainv, double*
             for (int k = i + 1; k < n; k++) s -= M[(long long)k * n + i] * Ainv[(long long)k * n + t];
             Ainv[(long long)i * n + t] = s / M[(long long)i * n + i];
         }
+        if (sizeof(T) == 4)
+            for (int i = 0; i < n; i++) put_inv<T>(Ainv, (long long)i * n + t, Ainv[(long long)i * n + t]);
     }
 }
 
@@ -412,11 +429,8 @@ __global__ void __launch_bounds__(128) k_coarse_apply(int n, const double* __res
                                                       T* __restrict__ z) {
     const int lane = threadIdx.x & 31;
     for (int i = (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += (int)(gridDim.x * blockDim.x) >> 5) {
-        const double* row = Ainv + (long long)i * n;
-        double s = 0.0;
-        for (int j = lane; j < n; j += 32) s += row[j] * (double)r[j];
-        s = warp_sum(s);
-        if (lane == 0) z[i] = (T)s;
+        const T v = coarse_row<32, T>(Ainv, n, i, lane, [&](int q) { return r[q]; });
+        if (lane == 0) z[i] = v;
     }
 }
 

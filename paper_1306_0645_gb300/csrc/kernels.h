@@ -188,7 +188,8 @@ template <class T>
 void launch_restrict(const Dims& f, const Dims& c, const T* rf, T* rc, cudaStream_t s);
 template <class T>
 void launch_prolong_add(const Dims& f, const Dims& c, const T* ec, T* zf, cudaStream_t s);
-// ---- coarsest grid (k_coarse.cu): the explicit inverse in ainv (FP64, n x n;
+// ---- coarsest grid (k_coarse.cu): the explicit inverse in ainv (n x n words
+// of 8 bytes: FP64 for T = double, a float pair high + low for T = float;
 // fp32: of FP32 accuracy up to 160 cells, else FP64 accuracy).  dense: n x n
 // FP64 words of scratch; flag: one word of scratch; a non-positive pivot
 // sets sc[S_BAD] = 2.
@@ -252,25 +253,37 @@ void launch_opacity_update(long long n, const double* E, const double* nH, const
 // in one launch of one cluster of `cluster` CTAs.  L[0].r is the input,
 // L[0].z the output; the other r, z, t are the levels' work vectors.
 constexpr int TAIL_MAX_LEVELS = 12;
-// small levels of the tail run in one CTA with their vectors (r, z, t) in
-// shared memory: from the first level with at most this many cells, when
-// their vectors fit TAIL_SMEM_MAX bytes
-constexpr long long TAIL_SMALL_CELLS = 512;
-constexpr size_t TAIL_SMEM_MAX = 160 * 1024;
+// levels of at most this many cells run in one CTA in shared memory
+constexpr long long TAIL_SOLO_CELLS = 4096;
+constexpr size_t TAIL_SMEM_MAX = 208 * 1024;
 template <class T>
 struct TailLevel {
     Dims d;
     Op<T> A;
     T *r, *z, *t;
+    int o_r, o_z, o_t, o_c, o_i;   // shared-memory offsets of a solo level's r, z,
+                                   // red residual, coefficients, pair table
 };
 template <class T>
 struct TailArgs {
     int nlev, pre, post;
     int paper_order;  // post-sweeps red then black (else black then red)
-    int small_from;   // first level run by one CTA in shared memory (nlev: none)
-    const double* ainv;
+    // filled by plan_tail:
+    int small_from;   // first level run by one CTA in shared memory
+    int slab;         // level run as halo slabs of the cluster's CTAs (-1: none)
+    int slab_axis;
+    int big_coarse;   // the coarsest grid is applied by the whole cluster
+    int coef_smem;    // solo coefficients in shared memory
+    int solve;        // layout of a whole inner solve by one CTA
+    int o_slab_r, o_slab_z, o_slab_t, o_slab_i, o_p, o_ainv;
+    int smem_bytes;
+    const double* ainv;   // coarsest inverse (see launch_coarse_setup)
     TailLevel<T> L[TAIL_MAX_LEVELS];
 };
+// Chooses how the levels run and the shared-memory layout for a cluster of
+// that many CTAs; false if it does not fit.
+template <class T>
+bool plan_tail(TailArgs<T>& a, int cluster, bool solve);
 template <class T>
 cudaError_t launch_vtail(const TailArgs<T>& a, int cluster, cudaStream_t s);
 // the cluster size to launch the tail with (16 or 8 CTAs), 0 if no cluster
@@ -288,14 +301,14 @@ struct PsReq {
     float *x, *p, *q;    // fine-level CG vectors
     double* sc;          // the request's scalar slots: S_THRESH, S_MAXIT in;
                          // S_KITER, S_RR, S_RHO.., S_NONFINITE out
-    int cta;             // 1: solved by one CTA with every vector in its
-                         // shared memory (psolve_cta_bytes fits), else by a cluster
+    int cta;             // 1: solved by one CTA with every level in its
+                         // shared memory (plan_tail with solve), else by a cluster
     int pad_;
 };
 constexpr int PS_MAX_BATCH = 256;
 constexpr int PS_CLUSTER = 8;
 // the most dynamic shared memory of a persistent launch
-constexpr size_t PS_SMEM_MAX = 200 * 1024;
+constexpr size_t PS_SMEM_MAX = 208 * 1024;
 struct PsBatch {
     int n;          // requests: [0, ncl) by clusters, [ncl, n) by single CTAs
     int ncl;
@@ -307,11 +320,8 @@ struct PsShape {
     int clusters;   // clusters resident at once
 };
 PsShape psolve_shape();
-// shared memory of a single-CTA solve: r, z, t of every level and p, q, x
-size_t psolve_cta_bytes(const TailArgs<float>& v);
-size_t psolve_smem_bytes(const PsReq& r);
 // one launch: min(n, resident clusters) clusters drain the work list; smem
-// is the largest psolve_smem_bytes of the batch
+// is the largest smem_bytes of the batch's plans
 cudaError_t launch_psolve(const PsBatch& b, size_t smem, cudaStream_t s);
 
 // Sets the calling thread's fld_last_error message (fld_api.cu).
