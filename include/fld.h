@@ -441,7 +441,8 @@ fld_status fld_autotune(fld_ctx* ctx, int reps);
 
 /* The tuning table: per level and kernel one record of three ints
  * (threads per block, a power of two in [32, 256]; target blocks in
- * [1, 9728]; L2 prefetch distance in planes, [0, 8]); its length
+ * [1, 9728]; L2 prefetch distance in planes, [0, 8]; the default record 256,
+ * 1216 leaves the shape to the library); its length
  * (3 x 7 kernels x levels), a copy, and a
  * replacement (for caching tuned shapes).  fld_set_tuning checks every
  * record and changes nothing on FLD_EINVAL; the launch shape never changes

@@ -63,14 +63,14 @@ enum KClass {
     K_ASM_FACES = 0, K_ASM_RHS, K_COARSEN, K_INVD, K_COARSE_SETUP, K_SMOOTH_ZERO,
     K_RB_COLOUR, K_JACOBI, K_RESIDUAL, K_RESTRICT, K_PROLONG, K_COARSE_APPLY, K_DOT,
     K_CG_PMATVEC, K_CG_UPDATE, K_RESIDUAL64, K_IR_SCALE, K_IR_UPDATE, K_FINALIZE, K_APPLY,
-    K_OPACITY, K_COARSE_LEVELS, K_ASM_FIX, K_POST_FUSED, K_VTAIL, K_IR_RESID, K_PSOLVE, K_NUM
+    K_OPACITY, K_COARSE_LEVELS, K_ASM_FIX, K_POST_FUSED, K_VTAIL, K_IR_RESID, K_PSOLVE, K_BLACK, K_NUM
 };
 const char* const KNAMES[K_NUM] = {
     "assemble_faces", "assemble_rhs", "coarsen", "invd", "coarse_setup", "smooth_zero",
     "rb_colour", "jacobi", "residual", "restrict", "prolong_add", "coarse_apply", "dot",
     "cg_p_matvec", "cg_update", "residual64", "ir_scale", "ir_update", "finalize", "apply",
     "opacity_update", "coarse_levels", "assemble_fix", "post_smooth", "vtail", "ir_residual",
-    "psolve"};
+    "psolve", "black_sweep"};
 
 struct KStat {
     long long launches, timed;
@@ -510,6 +510,13 @@ void prolong_any(const Dims& f, const Dims& c, const T* ec, T* zf, cudaStream_t 
     launch_prolong_add<T>(f, c, ec, zf, s);
 }
 
+// Whether level l (with bfloat16 coefficients, so one sweep down) runs the
+// red/black compressed sweeps: one symmetric sweep up, and eight cells per
+// thread.
+bool compressed_sweeps(const fld_ctx* c, int l) {
+    return c->p.post == 1 && !c->p.paper_order && c->L[l].Abf.wx && fine8_ok(c->L[l].d);
+}
+
 // z = B r on level l (zero initial guess).  If dot is given and the last
 // post-smoothing sweep of this level can carry it, <r, z> goes there (with
 // reduction *dot) and *dot_done is set.
@@ -558,6 +565,28 @@ void vcycle(fld_ctx* c, int l, const T* r, T* z, const RedArgs* dot = nullptr, b
     // of the face weights and the inverse diagonal
     const bool bf = std::is_same<T, float>::value && L.Abf.wx != nullptr;
     const double cw = bf ? 0.5 : 1.0;
+    if constexpr (std::is_same<T, float>::value) {
+        if (bf && compressed_sweeps(c, l)) {
+            // one colour at a time (k_fine8.cu): the red values in z's room
+            // until the last sweep writes z, the residual and the black
+            // values in the two halves of t
+            Level& C = c->L[l + 1];
+            const double nc = (double)C.d.n;
+            float* res = t;
+            float* zb = t + L.d.n / 2;
+            { KScope k(c, kc(K_SMOOTH_ZERO), 16.0 * n); launch_zero8(L.d, L.Abf, r, z, zb, s, L.tune[TN_SMOOTH0]); }
+            { KScope k(c, kc(K_RESIDUAL), 10.0 * n); launch_residual8(L.d, L.Abf, zb, res, s, L.tune[TN_RES]); }
+            { KScope k(c, kc(K_RESTRICT), 2.0 * n + 4.0 * nc);
+              launch_restrict4(L.d, C.d, res, (float*)C.r, s, L.tune[TN_RESTRICT], true); }
+            vcycle<float>(c, l + 1, (const float*)C.r, (float*)C.z);
+            { KScope k(c, kc(K_PROLONG), 4.0 * n + 4.0 * nc);
+              launch_correct8(L.d, C.d, (const float*)C.z, z, s, L.tune[TN_PROLONG]); }
+            { KScope k(c, kc(K_BLACK), 16.0 * n); launch_black8(L.d, L.Abf, r, z, zb, s, L.tune[TN_RB]); }
+            { KScope k(c, kc(K_RB_COLOUR), 18.0 * n); launch_red8(L.d, L.Abf, r, zb, z, dot, s, L.tune[TN_RB]); }
+            if (dot) *dot_done = true;
+            return;
+        }
+    }
     if (p.smoother == FLD_SMOOTH_RBGS) {
         if (p.pre >= 1) {
             KScope k(c, kc(K_SMOOTH_ZERO), (2.0 + 4.0 * cw) * n * ts);
@@ -2504,6 +2533,7 @@ fld_status fld_autotune(fld_ctx* c, int reps) {
         float* r = l == 0 ? (float*)c->cg[0] : (float*)L.r;
         float* z = l == 0 ? (float*)c->cg[1] : (float*)L.z;
         float* t = (float*)L.t;
+        const bool comp = compressed_sweeps(c, l);
         // sweep inputs need finite values only; results are discarded
         cudaMemsetAsync(r, 0, nb, s);
         cudaMemsetAsync(z, 0, nb, s);
@@ -2535,21 +2565,27 @@ fld_status fld_autotune(fld_ctx* c, int reps) {
                 // the sweeps the V-cycle launches: bfloat16 coefficients where
                 // the level has them
                 case TN_SMOOTH0:
-                    if (L.Abf.wx) launch_smooth_zero4(L.d, L.Abf, r, t, s, tn);
+                    if (comp) launch_zero8(L.d, L.Abf, r, t, t + L.d.n / 2, s, tn);
+                    else if (L.Abf.wx) launch_smooth_zero4(L.d, L.Abf, r, t, s, tn);
                     else launch_smooth_zero4(L.d, L.A32, r, t, s, tn);
                     break;
                 case TN_RB:
-                    if (L.Abf.wx) launch_rb_colour4(L.d, L.Abf, r, t, 0, s, tn);
+                    if (comp) launch_red8(L.d, L.Abf, r, t, z, nullptr, s, tn);
+                    else if (L.Abf.wx) launch_rb_colour4(L.d, L.Abf, r, t, 0, s, tn);
                     else launch_rb_colour4(L.d, L.A32, r, t, 0, s, tn);
                     break;
                 case TN_RES:
-                    if (L.Abf.wx) launch_residual4(L.d, L.Abf, z, t, s, tn, red_compress_ok(L.d));
+                    if (comp) launch_residual8(L.d, L.Abf, z, t, s, tn);
+                    else if (L.Abf.wx) launch_residual4(L.d, L.Abf, z, t, s, tn, red_compress_ok(L.d));
                     else launch_residual4(L.d, L.A32, r, z, t, s, tn, zg_cfg, zg_cfg && red_compress_ok(L.d));
                     break;
                 case TN_RESTRICT:
                     launch_restrict4(L.d, C.d, t, (float*)C.t, s, tn, zg_cfg && red_compress_ok(L.d));
                     break;
-                case TN_PROLONG: launch_prolong_add4(L.d, C.d, (const float*)C.z, t, s, tn); break;
+                case TN_PROLONG:
+                    if (comp) launch_correct8(L.d, C.d, (const float*)C.z, t, s, tn);
+                    else launch_prolong_add4(L.d, C.d, (const float*)C.z, t, s, tn);
+                    break;
                 case TN_POST: launch_post_smooth4(L.d, L.A32, r, z, t, nullptr, s, tn); break;
                 case TN_PMATVEC:
                     launch_cg_p_matvec4(L.d, L.A32, z, (const float*)c->cg[2], (float*)c->cg[3],

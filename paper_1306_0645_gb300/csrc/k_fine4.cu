@@ -984,7 +984,9 @@ bool fine4_ok(const Dims& d) { return d.nx % 4 == 0 && d.nx >= 16; }
 
 void launch_cg_p_matvec4(const Dims& d, Op<float> A, const float* z, const float* p_in, float* p_out,
                          float* q, const RedArgs& ra, cudaStream_t s, const Tune& tn, float* x) {
-    ColShape sh = shape4(d, tn);
+    Dims h = d;
+    h.nx = d.nx / 4;
+    const ColShape sh = sweep_shape(h, tn);
     k_cg_p_matvec4<<<sh.grid, sh.block, 0, s>>>(d, A, z, p_in, p_out, q, x, ra, tn.pf);
 }
 void launch_residual4(const Dims& d, Op<float> A, const float* r, const float* z, float* res,
@@ -1012,7 +1014,7 @@ void launch_restrict4(const Dims& f, const Dims& c, const float* rf, float* rc, 
     Dims h = c;
     if (red_compressed) {
         h.nx = c.nx / 4;
-        ColShape sh = col_shape(h, tn.threads, tn.target);
+        const ColShape sh = sweep_shape(h, tn);
         k_restrict_red4<<<sh.grid, sh.block, 0, s>>>(f, c, rf, rc, tn.pf);
         return;
     }

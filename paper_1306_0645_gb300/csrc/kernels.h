@@ -338,6 +338,35 @@ struct Tune {
     int target = 152 * 8;
     int pf = 1;             // L2 prefetch distance in planes (0: none; FP32 sweeps)
 };
+
+// Launch shape of a sweep whose threads tile h (x extent in threads).  The
+// default record stands for the library's own choice: z-chunks 14 planes long
+// where that leaves at least five blocks per SM (the last wave of two or three
+// per SM then costs little, and a chunk's first plane, which reads three
+// planes, is a small share), else 8, else 4 planes where 1.5 blocks per SM
+// remain, else one.  A fixed 152 x 8 blocks gave two and a half waves and
+// chunks of 52 to 128 planes at 512^3 and one or two planes at 128^3.
+// Measured per launch, fixed -> this rule: p/q 1024 -> 824 us, smoothing 447 ->
+// 411, residual 247 -> 215, black sweep 407 -> 340, red sweep 401 -> 369 at
+// 512^3; p/q 29 -> 25, smoothing 18.0 -> 15.6, red 20.9 -> 16.3 at 128^3
+// (longer chunks there: p/q 28 at 7 planes; shorter at 512^3: red 386 at 7,
+// smoothing 423).
+inline ColShape sweep_shape(const Dims& h, const Tune& tn) {
+    const Tune def;
+    if (tn.threads != def.threads || tn.target != def.target) return col_shape(h, tn.threads, tn.target);
+    const ColShape one = col_shape(h, def.threads, 1);
+    const long long xy = (long long)one.grid.x * one.grid.y;
+    long long blocks = xy * h.nz;
+    for (int kch : {14, 8, 4}) {
+        const long long b = xy * ((h.nz + kch - 1) / kch);
+        if (b >= (kch > 4 ? 152 * 5 : 152 * 3 / 2)) {
+            blocks = b;
+            break;
+        }
+    }
+    if (blocks > RED_MAX_BLOCKS) blocks = RED_MAX_BLOCKS;
+    return col_shape(h, def.threads, (int)blocks);
+}
 constexpr int TUNE_FIELDS = 3;      // entries of one tuning-table record
 constexpr int TUNE_PF_MAX = 8;
 
@@ -371,6 +400,23 @@ void launch_rb_colour4_dot(const Dims& d, Op<unsigned short> A, const float* r, 
                            const RedArgs& ra, cudaStream_t s, const Tune& tn = Tune{});
 void launch_residual4(const Dims& d, Op<unsigned short> A, const float* z, float* res, cudaStream_t s,
                       const Tune& tn, bool red_compressed);
+// ---- red/black compressed sweeps (k_fine8.cu): bfloat16 coefficients, one
+// sweep down and one up; need nx % 8 == 0.  zr, zb, res: n / 2 values, cell l
+// of the colour at l >> 1.
+bool fine8_ok(const Dims& d);
+// zr, zb: one red/black sweep from zero
+void launch_zero8(const Dims& d, Op<unsigned short> A, const float* r, float* zr, float* zb, cudaStream_t s,
+                  const Tune& tn);
+// res: its residual at the red cells (launch_restrict4's compressed form)
+void launch_residual8(const Dims& d, Op<unsigned short> A, const float* zb, float* res, cudaStream_t s,
+                      const Tune& tn);
+// zr += P ec at the red cells
+void launch_correct8(const Dims& f, const Dims& c, const float* ec, float* zr, cudaStream_t s, const Tune& tn);
+// zb from zr; then z (natural order) from zb, with <r, z> when dot is given
+void launch_black8(const Dims& d, Op<unsigned short> A, const float* r, const float* zr, float* zb, cudaStream_t s,
+                   const Tune& tn);
+void launch_red8(const Dims& d, Op<unsigned short> A, const float* r, const float* zb, float* z, const RedArgs* dot,
+                 cudaStream_t s, const Tune& tn);
 // B.wx, wy, wz, invd = the bfloat16 values nearest to A's (n a multiple of 4).
 void launch_op_to_bf16(long long n, Op<float> A, Op<unsigned short> B, cudaStream_t s);
 void launch_dot4(long long n, const float* a, const float* b, const RedArgs& ra, cudaStream_t s);
