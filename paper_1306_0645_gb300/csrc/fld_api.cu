@@ -586,6 +586,27 @@ void vcycle(fld_ctx* c, int l, const T* r, T* z, const RedArgs* dot = nullptr, b
             if (dot) *dot_done = true;
             return;
         }
+    } else {
+        if (p.smoother == FLD_SMOOTH_RBGS && p.pre == 1 && p.post >= 1 && pair_ok(L.d)) {
+            // a red/black pair per thread (k_pair.cu); the correction goes to
+            // the colour that the first post-sweep does not replace
+            Level& C = c->L[l + 1];
+            const double nc = (double)C.d.n;
+            const int first = p.paper_order ? 0 : 1;
+            { KScope k(c, kc(K_SMOOTH_ZERO), 6.0 * n * ts); launch_zero_pair(L.d, A, r, z, s); }
+            { KScope k(c, kc(K_RESIDUAL), 4.5 * n * ts); launch_residual_pair(L.d, A, z, t, s); }
+            { KScope k(c, kc(K_RESTRICT), (0.5 * n + nc) * ts); launch_restrict_pair(L.d, C.d, t, (T*)C.r, s); }
+            vcycle<T>(c, l + 1, (const T*)C.r, (T*)C.z);
+            { KScope k(c, kc(K_PROLONG), (2.0 * n + nc) * ts);
+              launch_correct_pair(L.d, C.d, (const T*)C.z, z, 1 - first, s); }
+            for (int q = 0; q < 2 * p.post; q++) {
+                const RedArgs* last = q == 2 * p.post - 1 ? dot : nullptr;
+                KScope k(c, kc(K_RB_COLOUR), 6.5 * n * ts);
+                launch_colour_pair(L.d, A, r, z, first ^ (q & 1), last, s);
+            }
+            if (dot) *dot_done = true;
+            return;
+        }
     }
     if (p.smoother == FLD_SMOOTH_RBGS) {
         if (p.pre >= 1) {
@@ -722,7 +743,8 @@ void pcg_iteration(fld_ctx* c, int cur, bool mirror = true) {
                 launch_cg_p_matvec4(L0.d, A, z, p[cur], p[cur ^ 1], q, red(c, R_ALPHA), c->s, L0.tune[TN_PMATVEC], x);
             else launch_cg_p_matvec<T>(L0.d, A, z, p[cur], p[cur ^ 1], q, red(c, R_ALPHA), c->s);
         } else {
-            launch_cg_p_matvec<T>(L0.d, A, z, p[cur], p[cur ^ 1], q, red(c, R_ALPHA), c->s);
+            if (pair_ok(L0.d)) launch_pq_pair(L0.d, A, z, p[cur], p[cur ^ 1], q, red(c, R_ALPHA), c->s);
+            else launch_cg_p_matvec<T>(L0.d, A, z, p[cur], p[cur ^ 1], q, red(c, R_ALPHA), c->s);
         }
     }
     {

@@ -188,6 +188,21 @@ template <class T>
 void launch_restrict(const Dims& f, const Dims& c, const T* rf, T* rc, cudaStream_t s);
 template <class T>
 void launch_prolong_add(const Dims& f, const Dims& c, const T* ec, T* zf, cudaStream_t s);
+// ---- FP64 sweeps, a red/black pair of cells per thread (k_pair.cu); need an
+// even x extent.  res: the residual at the red cells after a sweep from zero,
+// n / 2 values, cell l at l >> 1.
+bool pair_ok(const Dims& d);
+void launch_zero_pair(const Dims& d, Op<double> A, const double* r, double* z, cudaStream_t s);
+void launch_residual_pair(const Dims& d, Op<double> A, const double* z, double* res, cudaStream_t s);
+void launch_restrict_pair(const Dims& f, const Dims& c, const double* res, double* rc, cudaStream_t s);
+// z += P ec at the cells of colour col
+void launch_correct_pair(const Dims& f, const Dims& c, const double* ec, double* z, int col, cudaStream_t s);
+// one colour of a sweep, with <r, z> of the result when dot is given
+void launch_colour_pair(const Dims& d, Op<double> A, const double* r, double* z, int col, const RedArgs* dot,
+                        cudaStream_t s);
+void launch_pq_pair(const Dims& d, Op<double> A, const double* z, const double* p_in, double* p_out, double* q,
+                    const RedArgs& ra, cudaStream_t s);
+
 // ---- coarsest grid (k_coarse.cu): the explicit inverse in ainv (n x n words
 // of 8 bytes: FP64 for T = double, a float pair high + low for T = float;
 // fp32: of FP32 accuracy up to 160 cells, else FP64 accuracy).  dense: n x n
