@@ -143,7 +143,8 @@ typedef struct {
                                   down to the coarsest run as one persistent
                                   thread-block-cluster kernel per V-cycle
                                   (default 32768, at most 2^24; 0 = one
-                                  launch per sweep);
+                                  launch per sweep; FP64 precision starts it
+                                  at 4096 cells at most);
                                   same arithmetic as the per-level kernels */
     int paper_order;           /* red/black Gauss-Seidel: 0 (default) post-
                                   sweeps black then red, so the V-cycle is a

@@ -2134,8 +2134,9 @@ fld_status fld_create(fld_ctx** out, const fld_grid* g, const fld_params* p, voi
     // the coarsest one and a cluster of the tail kernel fits on the device
     c->tail_from = -1;
     if (p->tail_cells > 0 && p->smoother == FLD_SMOOTH_RBGS && c->nl >= 2) {
+        const int cells = c->mixed ? p->tail_cells : std::min(p->tail_cells, TAIL_CELLS64);
         int l0 = 0;
-        while (l0 < c->nl - 1 && c->L[l0].d.n > p->tail_cells) l0++;
+        while (l0 < c->nl - 1 && c->L[l0].d.n > cells) l0++;
         c->tail_cluster = c->mixed ? vtail_cluster<float>() : vtail_cluster<double>();
         if (l0 < c->nl - 1 && c->nl - l0 <= TAIL_MAX_LEVELS && c->tail_cluster > 0) c->tail_from = l0;
     }

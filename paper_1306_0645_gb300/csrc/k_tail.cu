@@ -1353,7 +1353,8 @@ cudaLaunchConfig_t tail_config(int cluster, cudaStream_t s, cudaLaunchAttribute*
 
 // Chooses how each level of the tail runs and lays out the shared memory.
 // Solo: from the first level of at most TAIL_SOLO_CELLS cells that fits
-// (4096: a 16^3 level's phases take 0.3 us there, and its operator 64 KB).
+// (4096: a 16^3 level's operator takes 64 KB); in FP64 512, since one SM's two
+// FP64 lanes take 50 us for a 16^3 level, halo slabs on eight SMs 15.
 // The level above it as a slab where Table 1's cycle (one sweep down, one up)
 // runs and its planes fit.  Any other level phase by phase over the cluster.
 // Coefficients move to shared memory in FP32 where they fit.  A coarsest grid
@@ -1417,7 +1418,7 @@ bool plan_tail(TailArgs<T>& a, int cluster, bool solve) {
         return off <= limit;
     };
     const bool one = a.pre == 1 && a.post == 1 && !a.paper_order;
-    const long long most = solve ? 2LL * PS_PAIRS * TAIL_THREADS : TAIL_SOLO_CELLS;
+    const long long most = solve ? 2LL * PS_PAIRS * TAIL_THREADS : sizeof(T) == 8 ? TAIL_SOLO_CELLS64 : TAIL_SOLO_CELLS;
     for (int ls = 0; ls < nl && (!solve || ls == 0); ls++) {
         if (ls < nl - 1 && a.L[ls].d.n > most) continue;
         for (int slab = ls > 0 && one && !solve ? ls - 1 : -1; slab >= -1; slab = slab >= 0 ? -1 : -2)

@@ -270,6 +270,10 @@ void launch_opacity_update(long long n, const double* E, const double* nH, const
 constexpr int TAIL_MAX_LEVELS = 12;
 // levels of at most this many cells run in one CTA in shared memory
 constexpr long long TAIL_SOLO_CELLS = 4096;
+constexpr long long TAIL_SOLO_CELLS64 = 512;   // FP64
+// the largest level of an FP64 tail: at 32^3 the 16 SMs of a cluster take 40 us
+// for a level whose six launches over the whole GPU take 27
+constexpr int TAIL_CELLS64 = 4096;
 constexpr size_t TAIL_SMEM_MAX = 208 * 1024;
 template <class T>
 struct TailLevel {
