@@ -173,13 +173,14 @@ __device__ __forceinline__ void red_finalize(const RedArgs& ra, const double* v)
 // block to arrive (atomic ticket, no waiting) sums all partials in block
 // order and runs the finaliser.  The order of the additions depends only on
 // the launch shape, never on block scheduling.
+// G blocks take part, this one as number bid (grid_reduce: all of the grid; a
+// launch may also hold several reductions, each with a counter and partials of
+// its own).
 template <int NV>
-__device__ __forceinline__ void grid_reduce(double (&v)[NV], const bool (&ismax)[NV],
-                                            const RedArgs& ra) {
+__device__ __forceinline__ void grid_reduce_of(double (&v)[NV], const bool (&ismax)[NV], const RedArgs& ra, int G,
+                                               int bid) {
     block_reduce<NV>(v, ismax);
     __shared__ bool last;
-    const int G = gridDim.x * gridDim.y * gridDim.z;
-    const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
     const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
     const int nthr = blockDim.x * blockDim.y * blockDim.z;
     if (tid == 0) {
@@ -222,6 +223,12 @@ __device__ __forceinline__ void grid_reduce(double (&v)[NV], const bool (&ismax)
         red_finalize(ra, w);
         *ra.counter = 0u;
     }
+}
+template <int NV>
+__device__ __forceinline__ void grid_reduce(double (&v)[NV], const bool (&ismax)[NV],
+                                            const RedArgs& ra) {
+    grid_reduce_of<NV>(v, ismax, ra, gridDim.x * gridDim.y * gridDim.z,
+                       blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z));
 }
 
 // Per-thread accumulator of a dot product.  FP64 data accumulate with FMA.

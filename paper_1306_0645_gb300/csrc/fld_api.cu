@@ -1333,6 +1333,13 @@ void assemble_faces_range(fld_ctx* c, const double* E, const double* nHI, const 
 void assemble_rhs_range(fld_ctx* c, const double* E, const double* nHI, const double* eta, int zb0, int nzb,
                         double frac, const RedArgs& ra) {
     Level& L0 = c->L[0];
+    if (L0.bnd.mask) {
+        // the weights of the Dirichlet faces in those planes
+        const AsmShape a = asm_shape(L0.d);
+        KScope k(c, K_ASM_RHS, 0.0);
+        launch_bnd_weights(L0.d, c->pd, E, nHI, L0.bnd, zb0 * a.kch,
+                           nzb < 0 ? L0.d.nz : std::min(L0.d.nz, (zb0 + nzb) * a.kch), c->s);
+    }
     if (c->mixed) {
         // reads E, n_HI, eta, the df weights and the FP32 mass term; writes
         // b and the FP32 inverse diagonal
@@ -1356,24 +1363,16 @@ fld_status assemble_coarse(fld_ctx* c) {
         Level& C = c->L[l];
         const double nf = (double)F.d.n, nc = (double)C.d.n;
         if (c->mixed) {
-            { KScope k(c, K_COARSEN, 16.0 * (nf + nc)); launch_coarsen<float>(F.d, C.d, F.A32, C.A32, s); }
-            for (int sd = 0; sd < 6; sd++)
-                if ((C.bnd.mask >> sd) & 1) {
-                    KScope k(c, K_COARSEN, 0.0);
-                    launch_coarsen_bnd<float>(F.d, C.d, sd, F.bnd, C.bnd, C.A32, s);
-                }
+            { KScope k(c, K_COARSEN, 16.0 * (nf + nc));
+              launch_coarsen<float>(F.d, C.d, F.A32, C.A32, F.bnd, C.bnd, s); }
             { KScope k(c, K_INVD, 20.0 * nc); launch_invd<float>(C.d, C.A32, C.A32, s); }
             if (C.Abf.wx) {
                 KScope k(c, K_INVD, 24.0 * nc);
                 launch_op_to_bf16(C.d.n, C.A32, C.Abf, s);
             }
         } else {
-            { KScope k(c, K_COARSEN, 32.0 * (nf + nc)); launch_coarsen<double>(F.d, C.d, F.A64, C.A64, s); }
-            for (int sd = 0; sd < 6; sd++)
-                if ((C.bnd.mask >> sd) & 1) {
-                    KScope k(c, K_COARSEN, 0.0);
-                    launch_coarsen_bnd<double>(F.d, C.d, sd, F.bnd, C.bnd, C.A64, s);
-                }
+            { KScope k(c, K_COARSEN, 32.0 * (nf + nc));
+              launch_coarsen<double>(F.d, C.d, F.A64, C.A64, F.bnd, C.bnd, s); }
             { KScope k(c, K_INVD, 40.0 * nc); launch_invd<double>(C.d, C.A64, C.A64, s); }
         }
     }
@@ -1507,21 +1506,19 @@ void finalize_any(fld_ctx* c, long long n, double* E, const double* dE, const do
     else launch_finalize(n, c->pd, E, dE, nHI, eta, E, ra, c->s);
 }
 
-// Photons through the Dirichlet faces of side sd (before E is overwritten).
-void bnd_outflow_any(fld_ctx* c, int sd, const double* E) {
-    const RedArgs ra = red(c, R_STORE2, S_OUT0 + sd, S_OUTABS0 + sd);
-    if (c->mixed) launch_bnd_outflow_mx(c->L[0].d, c->pd, sd, c->L[0].bnd, E, c->dE, ra, c->sc, c->s);
-    else launch_bnd_outflow(c->L[0].d, c->pd, sd, c->L[0].bnd, E, c->dE, ra, c->s);
+// Photons through the Dirichlet faces (before E is overwritten).
+void bnd_outflow_any(fld_ctx* c, const double* E) {
+    if (!c->L[0].bnd.mask) return;
+    KScope k(c, K_FINALIZE, 0.0);
+    const RedArgs ra = red(c, R_STORE2);
+    if (c->mixed) launch_bnd_outflow_mx(c->L[0].d, c->pd, c->L[0].bnd, E, c->dE, ra, c->sc, c->s);
+    else launch_bnd_outflow(c->L[0].d, c->pd, c->L[0].bnd, E, c->dE, ra, c->s);
 }
 
 void finalize_enqueue(fld_ctx* c, double* E, const double* nHI, const double* eta) {
     const long long n = c->L[0].d.n;
     // the flux through Dirichlet faces needs E^n, before the update below
-    for (int sd = 0; sd < 6; sd++)
-        if ((c->L[0].bnd.mask >> sd) & 1) {
-            KScope k(c, K_FINALIZE, 0.0);
-            bnd_outflow_any(c, sd, E);
-        }
+    bnd_outflow_any(c, E);
     { KScope k(c, K_FINALIZE, 40.0 * n); finalize_any(c, n, E, c->dE, nHI, eta, red(c, R_STORE7_FIN)); }
     cudaEventRecord(c->e1, c->s);
     cudaMemcpyAsync(c->h_sc, c->sc, NUM_SLOTS * sizeof(double), cudaMemcpyDeviceToHost, c->s);
@@ -1548,11 +1545,7 @@ fld_status copy_streams(fld_ctx* c) {
 fld_status finalize_enqueue_host(fld_ctx* c, double* E, const double* nHI, const double* eta, double* E_host) {
     const Dims& d = c->L[0].d;
     const long long nxy = (long long)d.nx * d.ny;
-    for (int sd = 0; sd < 6; sd++)
-        if ((c->L[0].bnd.mask >> sd) & 1) {
-            KScope k(c, K_FINALIZE, 0.0);
-            bnd_outflow_any(c, sd, E);
-        }
+    bnd_outflow_any(c, E);
     const int nch = std::min(8, d.nz);
     if (fld_status st = copy_streams(c)) return st;
     for (int q = 0; q < nch; q++)

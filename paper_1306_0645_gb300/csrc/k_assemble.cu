@@ -163,17 +163,15 @@ __global__ void __launch_bounds__(RED_THREADS) k_assemble_rhs(Dims d, PhysDev p,
             // Dirichlet faces of the box touching this cell
             const int ijk[3] = {i, j, k};
             const int nn[3] = {d.nx, d.ny, d.nz};
-            const double kc = nHI[c] * p.sigma;
             double wb_sum = 0.0;
 #pragma unroll
             for (int sd = 0; sd < 6; sd++) {
                 const int a = sd >> 1;
                 if (!((p.dmask >> sd) & 1) || ijk[a] != ((sd & 1) ? nn[a] - 1 : 0)) continue;
                 const double Eb = p.ebc[sd];
-                const double wb = 2.0 * p.dt_h2[a] * face_D(Eb, Ec, kc, kc, 0.5 * p.h[a], p);
                 const long long f = a == 0 ? j + (long long)d.ny * k
                                            : (a == 1 ? i + (long long)d.nx * k : i + (long long)d.nx * j);
-                bnd.w[bnd_offset(d, sd) + f] = wb;
+                const double wb = bnd.w[bnd_offset(d, sd) + f];
                 wb_sum += wb;
                 flux = fma(wb, Eb - Ec, flux);
             }
@@ -275,33 +273,54 @@ void launch_assemble_rhs(const Dims& d, const PhysDev& p, const double* E, const
 // face flux is w_b [theta (E^{n+1} - E_b) + (1 - theta)(E^n - E_b)] / theta
 // per unit volume, i.e. w_b (inv_theta (E^n - E_b) + dE) with the stored
 // (theta-scaled) w_b.
-__global__ void __launch_bounds__(RED_THREADS) k_bnd_outflow(Dims d, PhysDev p, int sd, Bnd bnd,
+__global__ void __launch_bounds__(RED_THREADS) k_bnd_outflow(Dims d, PhysDev p, Bnd bnd,
                                                             const double* __restrict__ E,
                                                             const double* __restrict__ dE, RedArgs ra) {
-    const int a = sd >> 1, hi = sd & 1;
+    const int sd = blockIdx.y;
+    if (!((bnd.mask >> sd) & 1)) return;
     const long long nf = bnd_side_size(d, sd);
     const long long off = bnd_offset(d, sd);
-    const long long nu = a == 0 ? d.ny : d.nx;
     const double Eb = p.ebc[sd];
     double acc[2] = {0.0, 0.0};
-    GRID_LOOP(f, nf) {
-        const long long u = f % nu, v = f / nu;
-        long long i, j, k;
-        if (a == 0) { i = hi ? d.nx - 1 : 0; j = u; k = v; }
-        else if (a == 1) { i = u; j = hi ? d.ny - 1 : 0; k = v; }
-        else { i = u; j = v; k = hi ? d.nz - 1 : 0; }
+    for (long long f = blockIdx.x * (long long)blockDim.x + threadIdx.x; f < nf; f += (long long)gridDim.x * blockDim.x) {
+        int i, j, k;
+        bnd_cell(d, sd, f, i, j, k);
         const long long c = i + (long long)d.nx * (j + (long long)d.ny * k);
         const double fl = bnd.w[off + f] * fma(p.inv_theta, E[c] - Eb, dE[c]);
         acc[0] += fl;
         acc[1] += fabs(fl);
     }
     const bool mx[2] = {false, false};
-    grid_reduce<2>(acc, mx, ra);
+    grid_reduce_of<2>(acc, mx, bnd_red(ra, sd), gridDim.x, blockIdx.x);
 }
 
-void launch_bnd_outflow(const Dims& d, const PhysDev& p, int sd, Bnd bnd, const double* E,
-                        const double* dE, const RedArgs& ra, cudaStream_t st) {
-    k_bnd_outflow<<<red_blocks(bnd_side_size(d, sd)), RED_THREADS, 0, st>>>(d, p, sd, bnd, E, dE, ra);
+void launch_bnd_outflow(const Dims& d, const PhysDev& p, Bnd bnd, const double* E, const double* dE,
+                        const RedArgs& ra, cudaStream_t st) {
+    k_bnd_outflow<<<dim3(bnd_blocks(d), 6), RED_THREADS, 0, st>>>(d, p, bnd, E, dE, ra);
+}
+
+// Limiter weights of the Dirichlet faces: E_b half a cell out, the cell's
+// opacity on both sides.
+__global__ void __launch_bounds__(128) k_bnd_weights(Dims d, PhysDev p, const double* __restrict__ E,
+                                                     const double* __restrict__ nHI, Bnd bnd, int k0, int k1) {
+    const int sd = blockIdx.y, a = sd >> 1;
+    if (!((bnd.mask >> sd) & 1)) return;
+    const long long nf = bnd_side_size(d, sd);
+    for (long long f = blockIdx.x * (long long)blockDim.x + threadIdx.x; f < nf; f += (long long)gridDim.x * blockDim.x) {
+        int i, j, k;
+        bnd_cell(d, sd, f, i, j, k);
+        if (k < k0 || k >= k1) continue;
+        const long long c = i + (long long)d.nx * (j + (long long)d.ny * k);
+        const double kc = nHI[c] * p.sigma;
+        bnd.w[bnd_offset(d, sd) + f] = 2.0 * p.dt_h2[a] * face_D(p.ebc[sd], E[c], kc, kc, 0.5 * p.h[a], p);
+    }
+}
+
+void launch_bnd_weights(const Dims& d, const PhysDev& p, const double* E, const double* nHI, Bnd bnd, int k0, int k1,
+                        cudaStream_t s) {
+    long long m = 0;
+    for (int sd = 0; sd < 6; sd += 2) m = bnd_side_size(d, sd) > m ? bnd_side_size(d, sd) : m;
+    k_bnd_weights<<<dim3(grid_blocks(m, 128), 6), 128, 0, s>>>(d, p, E, nHI, bnd, k0, k1);
 }
 
 __global__ void k_opacity_update(long long n, const double* __restrict__ E, const double* __restrict__ nH,

@@ -72,8 +72,14 @@ __device__ __forceinline__ T nbr_sum_prod(const Dims& d, const Op<T>& A, long lo
 // Rediscretised coarse operator in precision T (FP64 for the FP64 cycle;
 // FP32 from the FP32 operator for the mixed solver's cycle, which alone
 // reads the coarse levels there).
-template <class T>
-__global__ void k_coarsen(Dims f, Dims cd, Op<T> F, Op<T> C) {
+//
+// BND: also the coarse Dirichlet face weights, the sum of the 4 fine weights
+// across each coarse face / 16 as for interior faces.  The mean of the 8
+// children's m holds their boundary weights / 8 = 2 w_c; the rediscretised
+// mass term has w_c, so w_c is taken back off, side by side in order.  (One
+// launch per side and level took 97 us of a 1.5 ms step at 128 x 64 x 64.)
+template <class T, bool BND>
+__global__ void k_coarsen(Dims f, Dims cd, Op<T> F, Op<T> C, Bnd FB, Bnd CB) {
     COL_BEGIN(cd)
         const int I = i, J = j, K = k;
         const long long fx = f.nx, fxy = (long long)f.nx * f.ny;
@@ -94,36 +100,26 @@ __global__ void k_coarsen(Dims f, Dims cd, Op<T> F, Op<T> C) {
                 sy += F.wy[base + a + fxy * b];
                 sz += F.wz[base + a + fx * b];
             }
-        C.m[c] = ms * (T)0.125;
+        T mc = ms * (T)0.125;
+        if (BND) {
+            const int ijk[3] = {i, j, k}, nn[3] = {cd.nx, cd.ny, cd.nz};
+#pragma unroll
+            for (int sd = 0; sd < 6; sd++) {
+                const int a = sd >> 1;
+                if (!((CB.mask >> sd) & 1) || ijk[a] != ((sd & 1) ? nn[a] - 1 : 0)) continue;
+                const long long u = a == 0 ? j : i, v = a == 2 ? j : k;
+                const long long nuc = a == 0 ? cd.ny : cd.nx, nuf = 2 * nuc;
+                const long long f00 = bnd_offset(f, sd) + 2 * u + nuf * 2 * v;
+                const double wc =
+                    ((FB.w[f00] + FB.w[f00 + 1]) + (FB.w[f00 + nuf] + FB.w[f00 + nuf + 1])) * 0.0625;
+                CB.w[bnd_offset(cd, sd) + u + nuc * v] = wc;
+                mc = (T)(mc - wc);
+            }
+        }
+        C.m[c] = mc;
         C.wx[c] = sx * (T)0.0625;
         C.wy[c] = sy * (T)0.0625;
         C.wz[c] = sz * (T)0.0625;
-    }
-}
-
-// Coarse Dirichlet face weights of side sd: the sum of the 4 fine weights
-// across each coarse face / 16, as for interior faces.  k_coarsen set the
-// coarse mass term to the mean of the 8 children's m, which holds their
-// boundary weights / 8 = 2 w_c; the rediscretised mass term has w_c, so
-// w_c is taken back off.
-template <class T>
-__global__ void k_coarsen_bnd(Dims f, Dims cd, int sd, Bnd F, Bnd C, Op<T> CA) {
-    const int a = sd >> 1, hi = sd & 1;
-    const long long nfc = bnd_side_size(cd, sd);
-    const long long offc = bnd_offset(cd, sd), offf = bnd_offset(f, sd);
-    const long long nuc = a == 0 ? cd.ny : cd.nx;
-    const long long nuf = 2 * nuc;
-    GRID_LOOP(fc, nfc) {
-        const long long u = fc % nuc, v = fc / nuc;
-        const long long f00 = offf + 2 * u + nuf * 2 * v;
-        const double wc = ((F.w[f00] + F.w[f00 + 1]) + (F.w[f00 + nuf] + F.w[f00 + nuf + 1])) * 0.0625;
-        C.w[offc + fc] = wc;
-        long long i, j, k;
-        if (a == 0) { i = hi ? cd.nx - 1 : 0; j = u; k = v; }
-        else if (a == 1) { i = u; j = hi ? cd.ny - 1 : 0; k = v; }
-        else { i = u; j = v; k = hi ? cd.nz - 1 : 0; }
-        T& mc = CA.m[i + (long long)cd.nx * (j + (long long)cd.ny * k)];
-        mc = (T)(mc - wc);
     }
 }
 
@@ -281,13 +277,10 @@ __global__ void k_prolong_add(Dims f, Dims cd, const T* __restrict__ ec, T* __re
 static const int TPB = 256;
 
 template <class T>
-void launch_coarsen(const Dims& f, const Dims& c, Op<T> F, Op<T> C, cudaStream_t s) {
+void launch_coarsen(const Dims& f, const Dims& c, Op<T> F, Op<T> C, Bnd FB, Bnd CB, cudaStream_t s) {
     ColShape sh = col_shape(c);
-    k_coarsen<T><<<sh.grid, sh.block, 0, s>>>(f, c, F, C);
-}
-template <class T>
-void launch_coarsen_bnd(const Dims& f, const Dims& c, int sd, Bnd F, Bnd C, Op<T> CA, cudaStream_t st) {
-    k_coarsen_bnd<T><<<grid_blocks(bnd_side_size(c, sd), 256), 256, 0, st>>>(f, c, sd, F, C, CA);
+    if (CB.mask) k_coarsen<T, true><<<sh.grid, sh.block, 0, s>>>(f, c, F, C, FB, CB);
+    else k_coarsen<T, false><<<sh.grid, sh.block, 0, s>>>(f, c, F, C, FB, CB);
 }
 template <class T>
 void launch_invd(const Dims& d, Op<T> A, const Op<T>& src, cudaStream_t s) {
@@ -329,8 +322,7 @@ void launch_prolong_add(const Dims& f, const Dims& c, const T* ec, T* zf, cudaSt
 }
 #define INST(T)                                                                                    \
     template void launch_invd<T>(const Dims&, Op<T>, const Op<T>&, cudaStream_t);                   \
-    template void launch_coarsen<T>(const Dims&, const Dims&, Op<T>, Op<T>, cudaStream_t);           \
-    template void launch_coarsen_bnd<T>(const Dims&, const Dims&, int, Bnd, Bnd, Op<T>, cudaStream_t); \
+    template void launch_coarsen<T>(const Dims&, const Dims&, Op<T>, Op<T>, Bnd, Bnd, cudaStream_t); \
     template void launch_smooth_zero<T>(const Dims&, Op<T>, const T*, T*, cudaStream_t);            \
     template void launch_rb_colour<T>(const Dims&, Op<T>, const T*, T*, int, cudaStream_t);         \
     template void launch_jacobi<T>(const Dims&, Op<T>, const T*, const T*, T*, double, bool,        \

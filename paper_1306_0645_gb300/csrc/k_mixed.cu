@@ -446,7 +446,6 @@ __global__ void __launch_bounds__(256) k_asm_rhs_mx(Dims d, PhysDev p, const dou
             // Dirichlet faces of the box touching this cell: E_b half a cell out
             const int ijk[3] = {i, j, k};
             const int nn[3] = {d.nx, d.ny, d.nz};
-            const double kc = nc * p.sigma;
             df wb_sum = {0.0f, 0.0f};
             bool any = false;
 #pragma unroll
@@ -454,10 +453,9 @@ __global__ void __launch_bounds__(256) k_asm_rhs_mx(Dims d, PhysDev p, const dou
                 const int a = sd >> 1;
                 if (!((p.dmask >> sd) & 1) || ijk[a] != ((sd & 1) ? nn[a] - 1 : 0)) continue;
                 const double Eb = p.ebc[sd];
-                const double wb = 2.0 * p.dt_h2[a] * face_D(Eb, Ec, kc, kc, 0.5 * p.h[a], p);
                 const long long f = a == 0 ? j + (long long)d.ny * k
                                            : (a == 1 ? i + (long long)d.nx * k : i + (long long)d.nx * j);
-                bnd.w[bnd_offset(d, sd) + f] = wb;
+                const double wb = bnd.w[bnd_offset(d, sd) + f];
                 const df wbd = d2df_rn(wb);
                 F.add(df_mul_raw(wbd, split64(Eb - Ec, K)));
                 wb_sum = df_add(wb_sum, wbd);
@@ -1067,23 +1065,20 @@ __global__ void __launch_bounds__(RED_THREADS) k_finalize_mx(long long n, PhysDe
 
 // Photons through the Dirichlet faces of side sd over the step, as
 // k_bnd_outflow, with dE the df iterate scaled by 2^-K.
-__global__ void __launch_bounds__(RED_THREADS) k_bnd_outflow_mx(Dims d, PhysDev p, int sd, Bnd bnd,
+__global__ void __launch_bounds__(RED_THREADS) k_bnd_outflow_mx(Dims d, PhysDev p, Bnd bnd,
                                                                const double* __restrict__ E,
                                                                const float2* __restrict__ dE, RedArgs ra,
                                                                const double* scg) {
+    const int sd = blockIdx.y;
+    if (!((bnd.mask >> sd) & 1)) return;
     const int K = step_scale(scg, p.dt_exp);
-    const int a = sd >> 1, hi = sd & 1;
     const long long nf = bnd_side_size(d, sd);
     const long long off = bnd_offset(d, sd);
-    const long long nu = a == 0 ? d.ny : d.nx;
     const double Eb = p.ebc[sd];
     double acc[2] = {0.0, 0.0};
-    GRID_LOOP(f, nf) {
-        const long long u = f % nu, v = f / nu;
-        long long i, j, k;
-        if (a == 0) { i = hi ? d.nx - 1 : 0; j = u; k = v; }
-        else if (a == 1) { i = u; j = hi ? d.ny - 1 : 0; k = v; }
-        else { i = u; j = v; k = hi ? d.nz - 1 : 0; }
+    for (long long f = blockIdx.x * (long long)blockDim.x + threadIdx.x; f < nf; f += (long long)gridDim.x * blockDim.x) {
+        int i, j, k;
+        bnd_cell(d, sd, f, i, j, k);
         const long long c = i + (long long)d.nx * (j + (long long)d.ny * k);
         const float2 dv = dE[c];
         const double d64 = f2d(dv.x, K) + f2d(dv.y, K);
@@ -1092,7 +1087,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_bnd_outflow_mx(Dims d, PhysDev 
         acc[1] += fabs(fl);
     }
     const bool mx[2] = {false, false};
-    grid_reduce<2>(acc, mx, ra);
+    grid_reduce_of<2>(acc, mx, bnd_red(ra, sd), gridDim.x, blockIdx.x);
 }
 
 // ------------------------------------------------------------------ hooks
@@ -1260,10 +1255,9 @@ void launch_finalize_mx(long long n, const PhysDev& p, const double* E, const vo
                                                                     scg);
 }
 
-void launch_bnd_outflow_mx(const Dims& d, const PhysDev& p, int sd, Bnd bnd, const double* E, const void* dE,
+void launch_bnd_outflow_mx(const Dims& d, const PhysDev& p, Bnd bnd, const double* E, const void* dE,
                            const RedArgs& ra, const double* scg, cudaStream_t st) {
-    k_bnd_outflow_mx<<<red_blocks(bnd_side_size(d, sd)), RED_THREADS, 0, st>>>(d, p, sd, bnd, E, (const float2*)dE,
-                                                                              ra, scg);
+    k_bnd_outflow_mx<<<dim3(bnd_blocks(d), 6), RED_THREADS, 0, st>>>(d, p, bnd, E, (const float2*)dE, ra, scg);
 }
 
 void launch_df_to_f64(long long n, const float* h, const float* l, double* out, cudaStream_t s) {

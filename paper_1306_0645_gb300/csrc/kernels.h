@@ -65,6 +65,16 @@ __host__ __device__ inline long long bnd_offset(const Dims& d, int s) {
     return o;
 }
 
+// Cell (i, j, k) of face f (within side sd) of level d.
+__device__ __forceinline__ void bnd_cell(const Dims& d, int sd, long long f, int& i, int& j, int& k) {
+    const int a = sd >> 1, hi = sd & 1;
+    const unsigned nu = a == 0 ? d.ny : d.nx;
+    const int v = (int)((unsigned)f / nu), u = (int)((unsigned)f - (unsigned)v * nu);
+    if (a == 0) { i = hi ? d.nx - 1 : 0; j = u; k = v; }
+    else if (a == 1) { i = u; j = hi ? d.ny - 1 : 0; k = v; }
+    else { i = u; j = v; k = hi ? d.nz - 1 : 0; }
+}
+
 // Per-block lists of the faces the FP32 screen could not settle, finished
 // by a compacted FP64 pass.  entries == nullptr disables the lists.
 struct FaceList {
@@ -106,12 +116,35 @@ void face_list_shape(const Dims& d, int limiter, long long* blocks, int* cap);
 void launch_assemble_rhs(const Dims& d, const PhysDev& p, const double* E, const double* nHI,
                          const double* eta, Op<double> op, Op<float> op32, double* b, double* diag64,
                          Bnd bnd, const RedArgs& ra, cudaStream_t s, int zb0 = 0, int nzb = -1);
-// Photons through the Dirichlet faces of side s over the step (before the
-// finalisation overwrites E): sum of w_b (inv_theta (E - E_b) + dE) into
-// slot S_OUT0 + s and the sum of its absolute values into S_OUTABS0 + s
-// (reduction ra with op R_STORE2).
-void launch_bnd_outflow(const Dims& d, const PhysDev& p, int s, Bnd bnd, const double* E,
-                        const double* dE, const RedArgs& ra, cudaStream_t st);
+// The limiter weights of the Dirichlet faces of the cells in planes [k0, k1)
+// into bnd.w, all sides in one launch; launch_assemble_rhs and
+// launch_asm_rhs_mx read them.  (In the right-hand side's sweep, where the
+// face cells are one or two lanes of a warp, the FP64 limiter cost 57 of its
+// 82 us at 128 x 64 x 64.)
+void launch_bnd_weights(const Dims& d, const PhysDev& p, const double* E, const double* nHI, Bnd bnd, int k0, int k1,
+                        cudaStream_t s);
+// Photons through the Dirichlet faces over the step (before the finalisation
+// overwrites E): per side s the sum of w_b (inv_theta (E - E_b) + dE) into slot
+// S_OUT0 + s and the sum of its absolute values into S_OUTABS0 + s, all sides
+// in one launch (reduction ra with op R_STORE2; it uses the six counters and
+// partials after ra's).
+void launch_bnd_outflow(const Dims& d, const PhysDev& p, Bnd bnd, const double* E, const double* dE,
+                        const RedArgs& ra, cudaStream_t st);
+// Blocks per side of such a launch, and side sd's share of the reduction.
+constexpr int BND_MAX_BLOCKS = 1024;
+inline int bnd_blocks(const Dims& d) {
+    long long m = 0;
+    for (int s = 0; s < 6; s += 2) m = bnd_side_size(d, s) > m ? bnd_side_size(d, s) : m;
+    const int b = red_blocks(m);
+    return b < BND_MAX_BLOCKS ? b : BND_MAX_BLOCKS;
+}
+__device__ __forceinline__ RedArgs bnd_red(RedArgs ra, int sd) {
+    ra.partials += sd * BND_MAX_BLOCKS;
+    ra.counter += 1 + sd;
+    ra.slot0 = S_OUT0 + sd;
+    ra.slot1 = S_OUTABS0 + sd;
+    return ra;
+}
 
 // ---- mixed-precision step on the FP32 pipe in double-float arithmetic
 // (k_mixed.cu).  The fine operator is (A, L): the FP32 operator of the
@@ -155,7 +188,7 @@ ColShape ir_residual_shape(const Dims& d);
 void launch_finalize_mx(long long n, const PhysDev& p, const double* E, const void* dE, const double* nHI,
                         const double* eta, double* E_out, const RedArgs& ra, const double* scg, cudaStream_t s);
 // launch_bnd_outflow with dE the df x
-void launch_bnd_outflow_mx(const Dims& d, const PhysDev& p, int s, Bnd bnd, const double* E, const void* dE,
+void launch_bnd_outflow_mx(const Dims& d, const PhysDev& p, Bnd bnd, const double* E, const void* dE,
                            const RedArgs& ra, const double* scg, cudaStream_t st);
 // the df x as FP64 values (fld_solve's output)
 void launch_dE_to_f64(long long n, const void* x, double* out, const double* scg, int dt_exp, cudaStream_t s);
@@ -165,14 +198,11 @@ void launch_df_to_f64(long long n, const float* h, const float* l, double* out, 
 void launch_apply_mx(const Dims& d, Op<float> A, Op<float> L, const double* x, double* y, cudaStream_t s);
 
 // ---- multigrid (k_mg.cu), T = float or double
+// With Dirichlet faces (FB, CB) also the coarse face weights (sum of the 4
+// fine ones / 16); the coarse mass term, the mean of the children's full m,
+// gives back the difference: m_c -= w_c.
 template <class T>
-void launch_coarsen(const Dims& f, const Dims& c, Op<T> F, Op<T> C, cudaStream_t s);
-// Coarse Dirichlet face weights of side s (sum of the 4 fine ones / 16);
-// the coarse mass term, which k_coarsen took as the mean of the children's
-// full m, gives back the difference: m_c -= w_c.  After launch_coarsen.
-template <class T>
-void launch_coarsen_bnd(const Dims& f, const Dims& c, int s, Bnd F, Bnd C, Op<T> CA,
-                        cudaStream_t st);
+void launch_coarsen(const Dims& f, const Dims& c, Op<T> F, Op<T> C, Bnd FB, Bnd CB, cudaStream_t s);
 template <class T>
 void launch_invd(const Dims& d, Op<T> A, const Op<T>& src, cudaStream_t s);
 template <class T>
