@@ -577,7 +577,8 @@ void vcycle(fld_ctx* c, int l, const T* r, T* z, const RedArgs* dot = nullptr, b
             { KScope k(c, kc(K_SMOOTH_ZERO), 16.0 * n); launch_zero8(L.d, L.Abf, r, z, zb, s, L.tune[TN_SMOOTH0]); }
             { KScope k(c, kc(K_RESIDUAL), 10.0 * n); launch_residual8(L.d, L.Abf, zb, res, s, L.tune[TN_RES]); }
             { KScope k(c, kc(K_RESTRICT), 2.0 * n + 4.0 * nc);
-              launch_restrict4(L.d, C.d, res, (float*)C.r, s, L.tune[TN_RESTRICT], true); }
+              if (C.d.n <= RESTRICT_PAIR_CELLS) launch_restrict_pair<float>(L.d, C.d, res, (float*)C.r, s);
+              else launch_restrict4(L.d, C.d, res, (float*)C.r, s, L.tune[TN_RESTRICT], true); }
             vcycle<float>(c, l + 1, (const float*)C.r, (float*)C.z);
             { KScope k(c, kc(K_PROLONG), 4.0 * n + 4.0 * nc);
               launch_correct8(L.d, C.d, (const float*)C.z, z, s, L.tune[TN_PROLONG]); }
@@ -595,7 +596,7 @@ void vcycle(fld_ctx* c, int l, const T* r, T* z, const RedArgs* dot = nullptr, b
             const int first = p.paper_order ? 0 : 1;
             { KScope k(c, kc(K_SMOOTH_ZERO), 6.0 * n * ts); launch_zero_pair(L.d, A, r, z, s); }
             { KScope k(c, kc(K_RESIDUAL), 4.5 * n * ts); launch_residual_pair(L.d, A, z, t, s); }
-            { KScope k(c, kc(K_RESTRICT), (0.5 * n + nc) * ts); launch_restrict_pair(L.d, C.d, t, (T*)C.r, s); }
+            { KScope k(c, kc(K_RESTRICT), (0.5 * n + nc) * ts); launch_restrict_pair<T>(L.d, C.d, t, (T*)C.r, s); }
             vcycle<T>(c, l + 1, (const T*)C.r, (T*)C.z);
             { KScope k(c, kc(K_PROLONG), (2.0 * n + nc) * ts);
               launch_correct_pair(L.d, C.d, (const T*)C.z, z, 1 - first, s); }

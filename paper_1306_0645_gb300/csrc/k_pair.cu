@@ -192,9 +192,11 @@ __global__ void __launch_bounds__(256) k_sweep_pair(Dims d, Op<double> A, const 
 // Full weighting of a residual given at the red cells by pair (see
 // k_restrict): per fine row the red taps are 2I, 2I + 2 (even red) or 2I - 1,
 // 2I + 1, with weights 3/4 and 1/4; a tap folded onto a red boundary cell adds
-// to its weight.
-__global__ void __launch_bounds__(256) k_restrict_pair(Dims f, Dims cd, const double* __restrict__ t,
-                                                       double* __restrict__ rc) {
+// to its weight.  One coarse cell per thread: 32 independent loads, all but a
+// few of them L1 hits.
+template <class T>
+__global__ void __launch_bounds__(256) k_restrict_pair(Dims f, Dims cd, const T* __restrict__ t,
+                                                       T* __restrict__ rc) {
     COL_BEGIN(cd)
         const int nx2 = f.nx >> 1;
         auto tap = [](int I, int q, int n, int per) {
@@ -212,18 +214,18 @@ __global__ void __launch_bounds__(256) k_restrict_pair(Dims f, Dims cd, const do
             fj[q] = tap(j, q, f.ny, f.py);
             fk[q] = tap(k, q, f.nz, f.pz);
         }
-        double acc = 0.0;
+        T acc = T(0);
 #pragma unroll
         for (int a = 0; a < 4; a++) {
-            const double wa = a == 0 || a == 3 ? 0.25 : 0.75;
+            const T* plane = t + (long long)fk[a] * f.ny * nx2;
 #pragma unroll
             for (int b = 0; b < 4; b++) {
-                const double wt = wa * (b == 0 || b == 3 ? 0.25 : 0.75) * 0.125;
-                const long long row = ((long long)fk[a] * f.ny + fj[b]) * nx2;
+                const T wt = T((a == 0 || a == 3 ? 0.25 : 0.75) * (b == 0 || b == 3 ? 0.25 : 0.75) * 0.125);
+                const T* row = plane + fj[b] * nx2;
                 const bool o = ((fj[b] + fk[a]) & 1) != 0;
                 const bool end = !f.px && (o ? lo : hi), fold = !f.px && (o ? hi : lo);
-                acc = fma(fold ? wt : 0.75 * wt, t[row + i], acc);
-                acc = fma(end ? 0.0 : 0.25 * wt, t[row + (o ? im : ip)], acc);
+                acc = fma(fold ? wt : T(0.75) * wt, row[i], acc);
+                acc = fma(end ? T(0) : T(0.25) * wt, row[o ? im : ip], acc);
             }
         }
         rc[c] = acc;
@@ -349,10 +351,13 @@ void launch_residual_pair(const Dims& d, Op<double> A, const double* z, double* 
     const ColShape sh = shape_pair(d);
     k_sweep_pair<true, false><<<sh.grid, sh.block, 0, s>>>(d, A, nullptr, const_cast<double*>(z), res, 0, RedArgs{});
 }
-void launch_restrict_pair(const Dims& f, const Dims& c, const double* res, double* rc, cudaStream_t s) {
+template <class T>
+void launch_restrict_pair(const Dims& f, const Dims& c, const T* res, T* rc, cudaStream_t s) {
     const ColShape sh = col_shape(c, 128, 152 * 16);
-    k_restrict_pair<<<sh.grid, sh.block, 0, s>>>(f, c, res, rc);
+    k_restrict_pair<T><<<sh.grid, sh.block, 0, s>>>(f, c, res, rc);
 }
+template void launch_restrict_pair<float>(const Dims&, const Dims&, const float*, float*, cudaStream_t);
+template void launch_restrict_pair<double>(const Dims&, const Dims&, const double*, double*, cudaStream_t);
 void launch_correct_pair(const Dims& f, const Dims& c, const double* ec, double* z, int col, cudaStream_t s) {
     Dims h = f;
     h.nx = f.nx >> 1;

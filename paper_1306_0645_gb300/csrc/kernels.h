@@ -224,7 +224,15 @@ void launch_prolong_add(const Dims& f, const Dims& c, const T* ec, T* zf, cudaSt
 bool pair_ok(const Dims& d);
 void launch_zero_pair(const Dims& d, Op<double> A, const double* r, double* z, cudaStream_t s);
 void launch_residual_pair(const Dims& d, Op<double> A, const double* z, double* res, cudaStream_t s);
-void launch_restrict_pair(const Dims& f, const Dims& c, const double* res, double* rc, cudaStream_t s);
+// launch_restrict_pair also serves the FP32 cycle up to this many coarse cells:
+// a cell per thread there keeps the GPU full where four cells per thread
+// (launch_restrict4) leave it idle, and costs more instructions per cell.
+// A step of 64^3 (coarse 32^3) takes 951 us instead of 976, of 128x64x64 1244
+// instead of 1286; with the coarse 64^3 of 128^3 as well, one of 128^3 with
+// four groups 4434 instead of 4340, and of 512^3 57.2 ms instead of 53.9.
+constexpr long long RESTRICT_PAIR_CELLS = 131072;
+template <class T>
+void launch_restrict_pair(const Dims& f, const Dims& c, const T* res, T* rc, cudaStream_t s);
 // z += P ec at the cells of colour col
 void launch_correct_pair(const Dims& f, const Dims& c, const double* ec, double* z, int col, cudaStream_t s);
 // one colour of a sweep, with <r, z> of the result when dot is given
