@@ -7,13 +7,15 @@
 //    per thread.  A step publishes the pivot row and column in shared memory
 //    (two buffers, so one barrier per step) and updates every entry.  What
 //    bounds it is the serial chain of n steps (barrier, reciprocal, two
-//    shared-memory reads), about 90 cycles each: keeping the matrix in shared
-//    memory instead cost a division and a handful of shared-memory accesses
-//    per entry and a second barrier.
+//    shared-memory reads), 0.3 to 0.5 us each: 24 us at 64 cells, 64 at 128.
+//    Steps of 32 rows as below take 22 and 56 us, which a step of a 16^3
+//    or 128x64x64 grid does not show.
 //  - larger grids take elimination steps of 32 rows, one launch per step over
 //    64 x 64 tiles of the whole matrix (two copies, read and written in
-//    turn).  Every CTA inverts the 32 x 32 pivot block itself: about 2 us,
-//    less than another launch.
+//    turn).  Every CTA inverts the 32 x 32 pivot block itself, in the registers
+//    of one warp while the others load the tile, which costs less than another
+//    launch: a step of 693 cells takes 10.4 us, 13.5 with the inversion by the
+//    whole CTA and a barrier per row.
 // The mixed solver uses that FP32 inverse up to 160 cells.  The FP64 solver,
 // and the mixed one above 160 cells, refine it to FP64 column by column,
 // x += X32 (e - A x) with the residual in FP64 through the 7-point operator
@@ -168,6 +170,43 @@ __global__ void __launch_bounds__(S* S) k_gj_inverse(Dims d, Op<T> A, O* __restr
 
 // ---- blocked elimination, n > GJ_ONE_MAX
 
+// In-place inverse of a symmetric positive definite 32 x 32 matrix held by a
+// warp, row i of column `lane` in a[i], without pivoting: M'[k][j] = M[k][j] / p,
+// M'[i][j] = M[i][j] - f_i M'[k][j] with f_i = M[i][k], and 1 / p, -f_i / p in
+// column k.  Each step takes its pivot row from a[0] and shifts the rows by
+// one, so the loop stays rolled (32 steps leave them in place).  By symmetry
+// f_i is the pivot row's entry in column i (negated for i < k), so every lane
+// publishes one value and reads all 32 as eight vectors; with one shuffle per
+// f_i a step of the elimination of 693 cells took 11.6 us instead of 10.4.  The
+// next pivot row is published before the other rows are updated.  Returns false where a pivot was not positive (taken as
+// 1).
+__device__ __forceinline__ bool warp_invert(float (&a)[GB], float (&buf)[2][GB], int lane) {
+    bool ok = true;
+    buf[0][lane] = a[0];
+#pragma unroll 1
+    for (int k = 0; k < GB; k++) {
+        __syncwarp();
+        float f[GB];
+#pragma unroll
+        for (int q = 0; q < GB / 4; q++)
+            *reinterpret_cast<float4*>(f + 4 * q) = *reinterpret_cast<const float4*>(buf[k & 1] + 4 * q);
+        float p = f[0];
+        if (!(p > 0.0f)) {
+            ok = false;
+            p = 1.0f;
+        }
+        const float ip = 1.0f / p;
+        const bool own = lane == k;
+        const float rv = own ? ip : a[0] * ip;
+        a[0] = fmaf(-f[1], rv, own ? 0.0f : a[1]);
+        buf[(k + 1) & 1][(lane - k - 1) & 31] = lane < k + 1 ? -a[0] : a[0];
+#pragma unroll
+        for (int i = 2; i < GB; i++) a[i - 1] = fmaf(-f[i], rv, own ? 0.0f : a[i]);
+        a[GB - 1] = rv;
+    }
+    return ok;
+}
+
 // The dense matrix in FP32 (a warp per row); clears the flag.
 template <class T>
 __global__ void __launch_bounds__(256) k_dense32(Dims d, Op<T> A, float* __restrict__ M, unsigned* flag) {
@@ -192,29 +231,35 @@ __global__ void __launch_bounds__(256) k_gj_block(int n, int kb, const float* __
     __shared__ float P[GB][GB + 1];
     __shared__ float C[GT][GB + 1];     // M[i, kb]
     __shared__ float Rw[GB][GT + 1];    // M[kb, j], then t
-    __shared__ float buf[4 * GB];
+    __shared__ __align__(16) float buf[2][GB];
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int i0 = blockIdx.y * GT, j0 = blockIdx.x * GT;
-    float a[2][2];
+    float o[4][4];
 #pragma unroll
-    for (int q = 0; q < 2; q++)
+    for (int q = 0; q < 4; q++)
 #pragma unroll
-        for (int b = 0; b < 2; b++) {
-            const int i = kb + ty + 16 * q, j = kb + tx + 16 * b;
-            a[q][b] = i < n && j < n ? M[(long long)i * n + j] : (i == j ? 1.0f : 0.0f);
+        for (int b = 0; b < 4; b++) {
+            const int i = i0 + ty + 16 * q, j = j0 + tx + 16 * b;
+            const bool own = j >= kb && j < kb + GB;
+            o[q][b] = i < n && j < n && !own ? M[(long long)i * n + j] : 0.0f;
         }
-    for (int q = tid; q < GB * GT; q += 256) {
-        const int r = q / GT, j = j0 + q % GT;
-        Rw[r][q % GT] = kb + r < n && j < n ? M[(long long)(kb + r) * n + j] : 0.0f;
-        const int i = i0 + q / GB, cc = kb + q % GB;
-        C[q / GB][q % GB] = i < n && cc < n ? M[(long long)i * n + cc] : 0.0f;
+    if (tid < 32) {
+        float a[GB];
+#pragma unroll
+        for (int i = 0; i < GB; i++)
+            a[i] = kb + i < n && kb + tid < n ? M[(long long)(kb + i) * n + kb + tid] : (i == tid ? 1.0f : 0.0f);
+        const bool ok = warp_invert(a, buf, tid);
+        if (!ok && tid == 0) *flag = 1u;
+#pragma unroll
+        for (int i = 0; i < GB; i++) P[i][tid] = a[i];
+    } else {
+        for (int q = tid - 32; q < GB * GT; q += 224) {
+            const int r = q / GT, j = j0 + q % GT;
+            Rw[r][q % GT] = kb + r < n && j < n ? M[(long long)(kb + r) * n + j] : 0.0f;
+            const int i = i0 + q / GB, cc = kb + q % GB;
+            C[q / GB][q % GB] = i < n && cc < n ? M[(long long)i * n + cc] : 0.0f;
+        }
     }
-    const bool ok = gj_invert<16, 2>(a, GB, buf, tx, ty);
-    if (!ok && tid == 0) *flag = 1u;
-#pragma unroll
-    for (int q = 0; q < 2; q++)
-#pragma unroll
-        for (int b = 0; b < 2; b++) P[ty + 16 * q][tx + 16 * b] = a[q][b];
     __syncthreads();
     // t: rows ty + 16 q (q < 2), columns tx + 16 b (b < 4)
     float t[2][4] = {};
@@ -236,15 +281,6 @@ __global__ void __launch_bounds__(256) k_gj_block(int n, int kb, const float* __
         Rw[ty + 16][tx + 16 * b] = own ? P[ty + 16][jl] : t[1][b];
     }
     __syncthreads();
-    float o[4][4];
-#pragma unroll
-    for (int q = 0; q < 4; q++)
-#pragma unroll
-        for (int b = 0; b < 4; b++) {
-            const int i = i0 + ty + 16 * q, j = j0 + tx + 16 * b;
-            const bool own = j >= kb && j < kb + GB;
-            o[q][b] = i < n && j < n && !own ? M[(long long)i * n + j] : 0.0f;
-        }
     for (int m = 0; m < GB; m++) {
         float v[4];
 #pragma unroll
@@ -302,38 +338,50 @@ __device__ __forceinline__ void apply_row(const Dims& d, const Op<T>& A, int c, 
 // (e - A x) until the largest residual entry is at the rounding level of the
 // products it is formed from (2 diag |x| bounds every w_f (x - x_nbr) of a
 // neighbouring row).  Columns that stop improving before that, or need more
-// than REFINE_MAX corrections, raise the flag.
+// than REFINE_MAX corrections, raise the flag.  Bound by the L2 reads of X32
+// (all of it per CTA and correction) and the FP64 residual, so the columns are
+// spread evenly over the SMs, with a thread per row up to 768: 162 us at 693
+// cells and 13 at 64, where four columns per CTA of 256 threads took 276 us at
+// 693.
 constexpr int REFINE_MAX = 8;
+constexpr int REFINE_THREADS = 768;
+// entries of a row of r: room for vector loads
+constexpr int refine_row(int cb) { return cb == 3 ? 4 : (cb > 4 ? 8 : cb); }
 template <class T, int CB>
-__global__ void __launch_bounds__(256) k_coarse_refine(Dims d, Op<T> A, const float* __restrict__ X32,
-                                                       double* __restrict__ X, unsigned* flag) {
+__global__ void __launch_bounds__(REFINE_THREADS) k_coarse_refine(Dims d, Op<T> A, const float* __restrict__ X32,
+                                                                  double* __restrict__ X, unsigned* flag) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int n = (int)d.n;
+    constexpr int RB = refine_row(CB);
+    const int n = (int)d.n, nt = blockDim.x;
     double* x = reinterpret_cast<double*>(smem_raw);     // [n][CB]
-    float* r = reinterpret_cast<float*>(x + n * CB);     // [n][CB]
-    __shared__ double wmax[8], wscale[8];
+    float* r = reinterpret_cast<float*>(x + (n * CB + 1) / 2 * 2);     // [n][RB]
+    __shared__ double wscale[REFINE_THREADS / 32];
+    __shared__ float wmax[REFINE_THREADS / 32];
     const int c0 = blockIdx.x * CB;
-    for (int q = threadIdx.x; q < n * CB; q += 256) {
+    for (int q = threadIdx.x; q < n * CB; q += nt) {
         const int c = c0 + q % CB;
         x[q] = c < n ? (double)X32[(long long)(q / CB) * n + c] : 0.0;
     }
-    double prev = 1e300;
+    float prev = 1e30f;
     bool good = false;
     for (int it = 0;; it++) {
         __syncthreads();
-        double mx = 0.0, sc = 1.0;
-        for (int c = threadIdx.x; c < n; c += 256) {
+        float mx = 0.0f;
+        double sc = 1.0;
+        for (int c = threadIdx.x; c < n; c += nt) {
             double y[CB], dg;
             apply_row<T, CB>(d, A, c, x, y, dg);
 #pragma unroll
             for (int b = 0; b < CB; b++) {
                 const double e = c0 + b < n ? (c == c0 + b ? 1.0 : 0.0) - y[b] : 0.0;
-                r[c * CB + b] = (float)e;
-                mx = fmax(mx, isfinite(e) ? fabs(e) : 1e300);
+                const float e32 = (float)e;
+                r[c * RB + b] = e32;
+                mx = fmaxf(mx, isfinite(e32) ? fabsf(e32) : 1e30f);
                 sc = fmax(sc, 2.0 * dg * fabs(x[c * CB + b]));
             }
         }
-        mx = warp_max(mx);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_down_sync(0xffffffffu, mx, o));
         sc = warp_max(sc);
         if ((threadIdx.x & 31) == 0) {
             wmax[threadIdx.x >> 5] = mx;
@@ -342,30 +390,38 @@ __global__ void __launch_bounds__(256) k_coarse_refine(Dims d, Op<T> A, const fl
         __syncthreads();
         mx = wmax[0];
         sc = wscale[0];
-#pragma unroll
-        for (int q = 1; q < 8; q++) {
-            mx = fmax(mx, wmax[q]);
+        for (int q = 1; q < nt / 32; q++) {
+            mx = fmaxf(mx, wmax[q]);
             sc = fmax(sc, wscale[q]);
         }
-        good = mx <= 4.0 * 2.220446049250313e-16 * sc;
-        if (good || it >= REFINE_MAX || mx > 0.25 * prev) break;
+        good = (double)mx <= 4.0 * 2.220446049250313e-16 * sc;
+        if (good || it >= REFINE_MAX || mx > 0.25f * prev) break;
         prev = mx;
-        for (int i = threadIdx.x; i < n; i += 256) {
+        for (int i = threadIdx.x; i < n; i += nt) {
             float acc[CB];
 #pragma unroll
             for (int b = 0; b < CB; b++) acc[b] = 0.0f;
-#pragma unroll 8
+#pragma unroll 16
             for (int q = 0; q < n; q++) {
                 const float w = X32[(long long)q * n + i];
+                float rr[RB];
+                if constexpr (RB >= 4) {
 #pragma unroll
-                for (int b = 0; b < CB; b++) acc[b] = fmaf(w, r[q * CB + b], acc[b]);
+                    for (int v = 0; v < (CB + 3) / 4; v++)
+                        *reinterpret_cast<float4*>(rr + 4 * v) = *reinterpret_cast<const float4*>(r + q * RB + 4 * v);
+                } else {
+#pragma unroll
+                    for (int b = 0; b < CB; b++) rr[b] = r[q * RB + b];
+                }
+#pragma unroll
+                for (int b = 0; b < CB; b++) acc[b] = fmaf(w, rr[b], acc[b]);
             }
 #pragma unroll
             for (int b = 0; b < CB; b++) x[i * CB + b] += (double)acc[b];
         }
     }
     __syncthreads();
-    for (int q = threadIdx.x; q < n * CB; q += 256) {
+    for (int q = threadIdx.x; q < n * CB; q += nt) {
         const int c = c0 + q % CB;
         if (c < n) put_inv<T>(X, (long long)(q / CB) * n + c, x[q]);
     }
@@ -454,10 +510,13 @@ void gj_one(const Dims& d, Op<T> A, O* X, double* sc, unsigned* flag, cudaStream
 
 template <class T, int CB>
 void refine_go(const Dims& d, Op<T> A, const float* X32, double* X, unsigned* flag, cudaStream_t s) {
-    const size_t bytes = (size_t)d.n * CB * (sizeof(double) + sizeof(float));
+    const size_t x = ((size_t)d.n * CB + 1) / 2 * 2 * sizeof(double);
+    const size_t bytes = x + (size_t)d.n * refine_row(CB) * sizeof(float);
     auto kern = k_coarse_refine<T, CB>;
     if (bytes > 40 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    kern<<<(unsigned)((d.n + CB - 1) / CB), 256, bytes, s>>>(d, A, X32, X, flag);
+    const int rows = (int)(d.n + 31) / 32 * 32;
+    const int threads = rows < 256 ? 256 : (rows < REFINE_THREADS ? rows : REFINE_THREADS);
+    kern<<<(unsigned)((d.n + CB - 1) / CB), threads, bytes, s>>>(d, A, X32, X, flag);
 }
 
 }  // namespace
@@ -487,8 +546,14 @@ void launch_coarse_setup(const Dims& d, Op<T> A, double* dense, double* ainv, do
             other = t;
         }
     }
-    // columns per CTA: 4 while their x and r fit 96 KB
-    if (n <= 2048) refine_go<T, 4>(d, A, M, ainv, flag, s);
+    // columns per CTA: one wave of CTAs up to 5 columns each, beyond that 4
+    // while their x and r fit 96 KB (k_coarse_refine)
+    if (n <= 152) refine_go<T, 1>(d, A, M, ainv, flag, s);
+    else if (n <= 2 * 152) refine_go<T, 2>(d, A, M, ainv, flag, s);
+    else if (n <= 3 * 152) refine_go<T, 3>(d, A, M, ainv, flag, s);
+    else if (n <= 4 * 152) refine_go<T, 4>(d, A, M, ainv, flag, s);
+    else if (n <= 5 * 152) refine_go<T, 5>(d, A, M, ainv, flag, s);
+    else if (n <= 2048) refine_go<T, 4>(d, A, M, ainv, flag, s);
     else refine_go<T, 2>(d, A, M, ainv, flag, s);
     if (n <= 64) gj_go<T, double, double, 32, 2>(d, A, ainv, sc, nullptr, flag, s);
     else if (n <= GJ64_MAX) gj_go<T, double, double, 32, 4>(d, A, ainv, sc, nullptr, flag, s);

@@ -46,6 +46,7 @@ def dense(grid, m, w):
     ((4, 4, 2), (False,) * 3, 1), ((4, 4, 4), (False, True, False), 1), ((5, 13, 1), (False,) * 3, 1),
     ((4, 8, 4), (False,) * 3, 1), ((3, 43, 1), (False,) * 3, 1), ((4, 8, 5), (True,) * 3, 1),
     ((7, 23, 1), (False,) * 3, 1), ((9, 3, 7), (False, False, True), 1), ((11, 9, 7), (False,) * 3, 1),
+    ((19, 7, 3), (False, True, False), 1), ((11, 7, 7), (False,) * 3, 1),
     ((32, 32, 1), (False,) * 3, 1),
     # nearly singular: no FP32 inverse contracts the error, so the FP64
     # elimination replaces it (both its forms)
