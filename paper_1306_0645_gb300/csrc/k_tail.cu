@@ -321,8 +321,10 @@ __device__ void tail_up(const TailLevel<T>& L, Vec<T> v, const Dims& cd, const T
 // block barrier between phases.  A thread owns pairs of cells (2h, 2h + 1)
 // along x, one red and one black; a table per level holds what the phases need
 // of a pair's position (face flags, parities, coarse cell), so no phase
-// divides.  What bounds a phase is the latency of one barrier and two or three
-// dependent shared-memory reads, 0.2 to 0.4 us at up to 4096 cells.
+// divides.  A phase takes about 1.8 us at 16^3 and 0.5 us at 8^3: one SM's
+// instruction issue and fetch bound it (a 16^3 cycle is 84,600 warp
+// instructions, issued in a third of the cycles; the largest stall is for the
+// next instruction), not the barriers.
 //
 // z starts as r * invd at red cells (whoever produces r writes it), so the
 // first red/black sweep from zero is one black phase; the residual after it is

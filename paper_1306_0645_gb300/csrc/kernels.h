@@ -119,8 +119,8 @@ void launch_assemble_rhs(const Dims& d, const PhysDev& p, const double* E, const
 // The limiter weights of the Dirichlet faces of the cells in planes [k0, k1)
 // into bnd.w, all sides in one launch; launch_assemble_rhs and
 // launch_asm_rhs_mx read them.  (In the right-hand side's sweep, where the
-// face cells are one or two lanes of a warp, the FP64 limiter cost 57 of its
-// 82 us at 128 x 64 x 64.)
+// face cells are one or two lanes of a warp, the FP64 limiter cost 50 of its
+// 87 us at 128 x 64 x 64; this launch takes 8.)
 void launch_bnd_weights(const Dims& d, const PhysDev& p, const double* E, const double* nHI, Bnd bnd, int k0, int k1,
                         cudaStream_t s);
 // Photons through the Dirichlet faces over the step (before the finalisation
