@@ -366,8 +366,8 @@ inline int pow2ceil(int v) {
     return p;
 }
 
-inline ColShape col_shape(const Dims& d, int threads = 256, int target_blocks = 152 * 8) {
-    int bx = pow2ceil(d.nx) < 32 ? pow2ceil(d.nx) : 32;
+inline ColShape col_shape(const Dims& d, int threads = 256, int target_blocks = 152 * 8, int lanes = 32) {
+    int bx = pow2ceil(d.nx) < lanes ? pow2ceil(d.nx) : lanes;
     int by = threads / bx;
     if (by > pow2ceil(d.ny)) by = pow2ceil(d.ny);
     const int gx = (d.nx + bx - 1) / bx, gy = (d.ny + by - 1) / by;

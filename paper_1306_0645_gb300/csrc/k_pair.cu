@@ -333,12 +333,13 @@ __global__ void __launch_bounds__(256) k_pq_pair(Dims d, Op<double> A, const dou
 static ColShape shape_pair(const Dims& d) {
     Dims h = d;
     h.nx = d.nx >> 1;
-    const ColShape one = col_shape(h, 256, 1);
+    const int lanes = row_lanes(h);
+    const ColShape one = col_shape(h, 256, 1, lanes);
     const long long xy = (long long)one.grid.x * one.grid.y;
     long long blocks = xy * ((d.nz + 3) / 4);
     if (blocks < 152 * 2) blocks = xy * d.nz < 152 * 2 ? xy * d.nz : 152 * 2;
     if (blocks > RED_MAX_BLOCKS) blocks = RED_MAX_BLOCKS;
-    return col_shape(h, 256, (int)blocks);
+    return col_shape(h, 256, (int)blocks, lanes);
 }
 
 bool pair_ok(const Dims& d) { return d.nx % 2 == 0; }

@@ -396,6 +396,25 @@ struct Tune {
     int pf = 1;             // L2 prefetch distance in planes (0: none; FP32 sweeps)
 };
 
+// Lanes along x of a sweep's blocks, whose threads tile h: 16 or 8 where 32 (16)
+// would leave more than a tenth of them past the row's end (24 or 40 threads
+// in 32s leave 25 and 37 %; a row of 8 lanes of 16 bytes is still one line).
+// Only for launches that fill the GPU: below, the idle lanes cost nothing and
+// the extra row ends do.  Per launch at 320^3 (rows of 40 threads, p/q 80), 32
+// lanes -> this rule: smoothing 145 -> 123 us, residual 77 -> 67, black sweep
+// 106 -> 96, red 139 -> 120, correction 58 -> 42, restriction 66 -> 46, p/q 233
+// -> 220.
+constexpr long long ROW_LANES_MIN = 1 << 18;
+inline int row_lanes(const Dims& h) {
+    int lanes = 32;
+    if ((long long)h.nx * h.ny * h.nz < ROW_LANES_MIN) return lanes;
+    for (int b : {16, 8}) {
+        const int now = (h.nx + lanes - 1) / lanes * lanes, less = (h.nx + b - 1) / b * b;
+        if (10 * less < 9 * now) lanes = b;
+    }
+    return lanes;
+}
+
 // Launch shape of a sweep whose threads tile h (x extent in threads).  The
 // default record stands for the library's own choice: z-chunks 14 planes long
 // where that leaves at least five blocks per SM (the last wave of two or three
@@ -410,8 +429,9 @@ struct Tune {
 // smoothing 423).
 inline ColShape sweep_shape(const Dims& h, const Tune& tn) {
     const Tune def;
-    if (tn.threads != def.threads || tn.target != def.target) return col_shape(h, tn.threads, tn.target);
-    const ColShape one = col_shape(h, def.threads, 1);
+    const int lanes = row_lanes(h);
+    if (tn.threads != def.threads || tn.target != def.target) return col_shape(h, tn.threads, tn.target, lanes);
+    const ColShape one = col_shape(h, def.threads, 1, lanes);
     const long long xy = (long long)one.grid.x * one.grid.y;
     long long blocks = xy * h.nz;
     for (int kch : {14, 8, 4}) {
@@ -422,7 +442,7 @@ inline ColShape sweep_shape(const Dims& h, const Tune& tn) {
         }
     }
     if (blocks > RED_MAX_BLOCKS) blocks = RED_MAX_BLOCKS;
-    return col_shape(h, def.threads, (int)blocks);
+    return col_shape(h, def.threads, (int)blocks, lanes);
 }
 constexpr int TUNE_FIELDS = 3;      // entries of one tuning-table record
 constexpr int TUNE_PF_MAX = 8;

@@ -29,7 +29,7 @@ def dev(a):
 @pytest.mark.parametrize("n,periodic,dirichlet", [
     ((16, 12, 20), (0, 0, 0), False), ((16, 16, 16), (1, 1, 1), False), ((24, 20, 28), (1, 0, 0), False),
     ((40, 6, 10), (0, 1, 0), False), ((272, 8, 12), (0, 0, 1), False), ((288, 12, 8), (1, 0, 0), False),
-    ((48, 80, 16), (0, 1, 1), False), ((64, 64, 64), (0, 0, 0), True), ((128, 96, 160), (0, 0, 0), False)])
+    ((48, 80, 16), (0, 1, 1), False), ((192, 96, 128), (0, 0, 0), False), ((320, 96, 80), (1, 1, 0), False), ((64, 64, 64), (0, 0, 0), True), ((128, 96, 160), (0, 0, 0), False)])
 def test_compressed_cycle_is_symmetric(fld, n, periodic, dirichlet):
     case = synth.random_case(n, seed=51, periodic=tuple(map(bool, periodic)))
     if dirichlet:
