@@ -52,13 +52,14 @@ UNIT = "cell-solves/s"
 MODEL_ASM, MODEL_ITER, MODEL_IR, MODEL_FIN = 80.0, 144.0, 52.0, 24.0
 
 TRAFFIC_OVER_ALGORITHMIC = {
-    "rb_colour": 19.9 / 18.0,
-    "cg_p_matvec": 40.5 / 40.0,
-    "smooth_zero": 16.1 / 16.0,
-    "residual": 12.0 / 12.0,
-    "restrict": 2.1 / 2.5,
-    "prolong_add": 6.7 / 8.5,
-    "cg_update": 10.5 / 12.0,
+    "rb_colour": 18.0 / 18.0,
+    "black_sweep": 16.7 / 16.0,
+    "cg_p_matvec": 40.3 / 40.0,
+    "smooth_zero": 16.5 / 16.0,
+    "residual": 10.2 / 10.0,
+    "restrict": 2.0 / 2.5,
+    "prolong_add": 2.7 / 4.5,
+    "cg_update": 10.4 / 12.0,
 }
 
 
@@ -380,8 +381,7 @@ def main():
     traffic = ratio * bytes_per if ratio else None
     roofline = {"kernel": d["name"], "bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "traffic": traffic, "peak_kind": peak_kind,
-                # the DRAM bytes the launch moves (ncu ratio x algorithmic) over its time: a colour
-                # sweep changes half of z but writes every 16-byte group of it back
+                # the DRAM bytes the launch moves (ncu ratio x algorithmic) over its time
                 "traffic_frac": (traffic / (avg_ms * 1e-3) / 1e9 / peak) if traffic else None,
                 "launches_timed": d["timed"], "avg_launch_ms": avg_ms, "bytes_per_launch": bytes_per,
                 "share_of_step": d["ms"] / cal_ms,
