@@ -175,13 +175,15 @@ __global__ void __launch_bounds__(256, 3) k_zero8(Dims d, Op<unsigned short> A, 
     uint4 iv = ldc8(invd, p + g.c);
     uint4 wzc = ldc8(A.wz, p + g.c);
     for (int k = w.k0; k < w.k1; k++) {
-        if (pf > 0 && k + pf < w.k1) {
-            const long long q = p + g.c + (long long)pf * w.nxy;
-            pf2(r, q + w.nxy);
-            pf2(invd, q + w.nxy);
-            pf2(A.wx, q);
-            pf2(A.wy, q);
-            pf2(A.wz, q + w.nxy);
+        const long long ahead = p + g.c + (long long)pf * w.nxy;
+        if (pf_here(k, pf, w.k1)) {
+            pf2(A.wx, ahead);
+            pf2(A.wy, ahead);
+        }
+        if (pf_above(k, pf, w.k1, d.nz)) {
+            pf2(r, ahead + w.nxy);
+            pf2(invd, ahead + w.nxy);
+            pf2(A.wz, ahead + w.nxy);
         }
         const long long up = zup(d, k, w.nxy);
         const bool has_zu = k < d.nz - 1 || d.pz;
@@ -248,16 +250,18 @@ __global__ void __launch_bounds__(256, MODE == S_FINAL ? 3 : 4)
         float4 ud = ld4(u, (p + g.c + zdn(d, w.k0, w.nxy)) >> 1);
         uint4 wzc = ldc8(A.wz, p + g.c);
         for (int k = w.k0; k < w.k1; k++) {
-            if (pf > 0 && k + pf < w.k1) {
-                const long long q = p + g.c + (long long)pf * w.nxy;
-                pf2(u, (q + w.nxy) >> 1);
+            const long long ahead = p + g.c + (long long)pf * w.nxy;
+            if (pf_here(k, pf, w.k1)) {
                 if (MODE != S_RES) {
-                    pf2(r, q);
-                    pf2(A.invd, q);
+                    pf2(r, ahead);
+                    pf2(A.invd, ahead);
                 }
-                pf2(A.wx, q);
-                pf2(A.wy, q);
-                pf2(A.wz, q + w.nxy);
+                pf2(A.wx, ahead);
+                pf2(A.wy, ahead);
+            }
+            if (pf_above(k, pf, w.k1, d.nz)) {
+                pf2(u, (ahead + w.nxy) >> 1);
+                pf2(A.wz, ahead + w.nxy);
             }
             const long long up = zup(d, k, w.nxy);
             const bool has_zu = k < d.nz - 1 || d.pz;
@@ -377,7 +381,7 @@ __global__ void __launch_bounds__(256, 3) k_correct8(Dims f, Dims cd, const floa
             bp = row(wrap(K + 1, cd.nz, cd.pz), J1);
         }
         const long long h = ((long long)k * w.nxy + (long long)w.j * f.nx + 8 * w.i8) >> 1;
-        if (pf > 0 && k + pf < w.k1) pf2(zr, h + (((long long)pf * w.nxy) >> 1));
+        if (pf_here(k, pf, w.k1)) pf2(zr, h + (((long long)pf * w.nxy) >> 1));
         const int o = (w.j + k) & 1;      // parity of the red cells
         const bool odd = (k & 1) != 0;
         const float4 A0 = xs(a0, o), B0 = xs(b0, o);

@@ -26,6 +26,14 @@ __device__ __forceinline__ void pf2(const T* p, long long i) {
     asm volatile("prefetch.global.L2 [%0];" ::"l"(__cvta_generic_to_global(p + i)));
 }
 
+// Whether a walk of planes [.., k1) prefetches plane k + pf while it computes
+// plane k, and, of arrays it reads one plane ahead, plane k + pf + 1: a plane
+// past the grid's nz is never named, since it lies past the array's end.
+__host__ __device__ __forceinline__ bool pf_here(int k, int pf, int k1) { return pf > 0 && k + pf < k1; }
+__host__ __device__ __forceinline__ bool pf_above(int k, int pf, int k1, int nz) {
+    return pf_here(k, pf, k1) && k + pf + 1 < nz;
+}
+
 // Geometry of one 4-cell vector on one plane.  Indices of missing
 // neighbours (zero-gradient boundary) point at the cell itself; the matching
 // face weights are zero, so those values never contribute.

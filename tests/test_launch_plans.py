@@ -1,0 +1,50 @@
+"""Launch shapes and prefetch ranges that the library's headers compute on the
+host: a small program with the library's own inline functions is compiled and
+run here (no GPU)."""
+import os
+import subprocess
+
+import pytest
+
+from paper_1306_0645_gb300 import build
+
+# Every plane a walk names (own plane, and one above it) must lie in the grid.
+PREFETCH = r"""
+for (int nz = 1; nz <= 70; nz++)
+    for (int gz = 1; gz <= nz; gz++) {
+        const int kch = (nz + gz - 1) / gz;
+        for (int pf = 0; pf <= fld::TUNE_PF_MAX; pf++)
+            for (int b = 0; b < gz; b++) {
+                const int k0 = b * kch, k1 = nz < k0 + kch ? nz : k0 + kch;
+                for (int k = k0; k < k1; k++) {
+                    int top = -1;
+                    if (fld::pf_here(k, pf, k1)) top = k + pf;
+                    if (fld::pf_above(k, pf, k1, nz)) top = k + pf + 1;
+                    if (top >= nz) return fail("plane", nz, gz, pf, k);
+                    if (pf == 0 && top >= 0) return fail("prefetch off", nz, gz, pf, k);
+                    // and every plane but the first pf + 1 of a chunk is named
+                    if (pf > 0 && k + pf + 1 < k1 && top != k + pf + 1) return fail("missed", nz, gz, pf, k);
+                }
+            }
+    }
+"""
+
+
+def run_host(tmp_path, body):
+    """Compiles body into a program with the library's headers and runs it."""
+    src = tmp_path / "plan.cu"
+    src.write_text('#include <cstdio>\n#include "walk4.cuh"\n'
+                   "static int fail(const char* what, int a, int b, int c, int d) {\n"
+                   '    printf("%s: %d %d %d %d\\n", what, a, b, c, d);\n    return 1;\n}\n'
+                   "int main() {\n" + body + "    return 0;\n}\n")
+    exe = str(tmp_path / "plan")
+    cmd = [build.nvcc()] + build.ARCH + ["-O1", "-std=c++17", "--expt-relaxed-constexpr", "-I", build.INCLUDE, "-I",
+                                         build.CSRC, str(src), "-o", exe]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    r = subprocess.run([exe], capture_output=True, text=True, env=dict(os.environ, CUDA_VISIBLE_DEVICES=""))
+    assert r.returncode == 0, r.stdout
+
+
+def test_prefetched_planes_lie_in_the_grid(tmp_path):
+    run_host(tmp_path, PREFETCH)
