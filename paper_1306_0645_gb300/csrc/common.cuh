@@ -370,6 +370,9 @@ inline ColShape col_shape(const Dims& d, int threads = 256, int target_blocks = 
     int bx = pow2ceil(d.nx) < lanes ? pow2ceil(d.nx) : lanes;
     int by = threads / bx;
     if (by > pow2ceil(d.ny)) by = pow2ceil(d.ny);
+    // whole warps: the kernels' shuffles and sums take all 32 lanes, and lanes
+    // that do not exist give undefined values (rows past ny own no cell)
+    if (bx * by < 32) by = 32 / bx;
     const int gx = (d.nx + bx - 1) / bx, gy = (d.ny + by - 1) / by;
     long long xy = (long long)gx * gy;
     long long gz = (target_blocks + xy - 1) / xy;

@@ -29,6 +29,28 @@ for (int nz = 1; nz <= 70; nz++)
     }
 """
 
+# Blocks of a stencil sweep: whole warps whatever the extents, the plane
+# covered, no more blocks than the reductions hold partial sums for.
+SHAPES = r"""
+const int ny_[] = {1, 2, 3, 4, 5, 7, 8, 12, 16, 33, 96, 1000};
+for (int nx = 1; nx <= 140; nx++)
+    for (int ny : ny_)
+        for (int nz : {1, 2, 3, 8, 30, 200})
+            for (int threads : {32, 64, 128, 256})
+                for (int lanes : {8, 16, 32}) {
+                    fld::Dims d;
+                    d.nx = nx; d.ny = ny; d.nz = nz; d.px = d.py = d.pz = 0;
+                    d.n = (long long)nx * ny * nz;
+                    const fld::ColShape s = fld::col_shape(d, threads, 152 * 8, lanes);
+                    const int n = s.block.x * s.block.y * s.block.z;
+                    if (n % 32 || n > threads) return fail("block", nx, ny, threads, n);
+                    if ((int)(s.block.x * s.grid.x) < nx || (int)(s.block.y * s.grid.y) < ny)
+                        return fail("plane", nx, ny, threads, lanes);
+                    if ((long long)s.grid.x * s.grid.y * s.grid.z > fld::RED_MAX_BLOCKS || (int)s.grid.z > nz)
+                        return fail("blocks", nx, ny, nz, threads);
+                }
+"""
+
 
 def run_host(tmp_path, body):
     """Compiles body into a program with the library's headers and runs it."""
@@ -48,3 +70,7 @@ def run_host(tmp_path, body):
 
 def test_prefetched_planes_lie_in_the_grid(tmp_path):
     run_host(tmp_path, PREFETCH)
+
+
+def test_sweep_blocks_are_whole_warps(tmp_path):
+    run_host(tmp_path, SHAPES)
