@@ -490,11 +490,16 @@ __global__ void __launch_bounds__(128) k_coarse_apply(int n, const double* __res
     }
 }
 
+// A kernel's limit of dynamic shared memory belongs to the function and is
+// shared by every host thread, so each instantiation only ever sets the most
+// it can need (never this call's size: another thread's smaller grid would
+// lower it between this call and its launch).
 template <class T, class R, class O, int S, int PT>
 void gj_go(const Dims& d, Op<T> A, O* X, double* sc, unsigned* flag, const unsigned* only_if, cudaStream_t s) {
+    constexpr size_t most = (size_t)S * PT * S * PT * sizeof(R);
     const size_t bytes = (size_t)d.n * (size_t)d.n * sizeof(R);
     auto kern = k_gj_inverse<T, R, O, S, PT>;
-    if (bytes > 40 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (bytes > 40 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     kern<<<1, S * S, bytes, s>>>(d, A, X, sc, flag, only_if);
 }
 
@@ -508,12 +513,14 @@ void gj_one(const Dims& d, Op<T> A, O* X, double* sc, unsigned* flag, cudaStream
     else gj_go<T, float, O, 32, 5>(d, A, X, sc, flag, nullptr, s);
 }
 
+// x and r of CB columns (launch_coarse_setup chooses CB so that they fit)
+constexpr size_t REFINE_SMEM = 96 * 1024;
 template <class T, int CB>
 void refine_go(const Dims& d, Op<T> A, const float* X32, double* X, unsigned* flag, cudaStream_t s) {
     const size_t x = ((size_t)d.n * CB + 1) / 2 * 2 * sizeof(double);
     const size_t bytes = x + (size_t)d.n * refine_row(CB) * sizeof(float);
     auto kern = k_coarse_refine<T, CB>;
-    if (bytes > 40 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (bytes > 40 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)REFINE_SMEM);
     const int rows = (int)(d.n + 31) / 32 * 32;
     const int threads = rows < 256 ? 256 : (rows < REFINE_THREADS ? rows : REFINE_THREADS);
     kern<<<(unsigned)((d.n + CB - 1) / CB), threads, bytes, s>>>(d, A, X32, X, flag);

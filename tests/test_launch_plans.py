@@ -52,10 +52,41 @@ for (int nx = 1; nx <= 140; nx++)
 """
 
 
-def run_host(tmp_path, body):
-    """Compiles body into a program with the library's headers and runs it."""
+# The shared-memory limits that the coarsest grid's launchers set, recorded in
+# place of the runtime call (the launches themselves find no device).
+RECORD = r"""
+#include <map>
+#include <cuda_runtime.h>
+static std::map<const void*, int> g_limit;
+static int g_lowered = 0;
+template <class F>
+static cudaError_t record_limit(F* f, cudaFuncAttribute, int bytes) {
+    auto it = g_limit.emplace((const void*)f, bytes).first;
+    if (it->second != bytes) g_lowered = 1;
+    return cudaSuccess;
+}
+#define cudaFuncSetAttribute record_limit
+#include "k_coarse.cu"
+"""
+LIMITS = r"""
+for (int n : {64, 102, 125, 128, 130, 150, 160, 161, 300, 609, 693, 702, 760, 761, 854, 1024, 2048, 2049, 4096}) {
+    fld::Dims d;
+    d.nx = n; d.ny = d.nz = 1; d.px = d.py = d.pz = 0; d.n = n;
+    for (bool fp32 : {false, true}) {
+        fld::launch_coarse_setup<float>(d, fld::Op<float>{}, nullptr, nullptr, nullptr, nullptr, fp32, nullptr);
+        if (g_lowered) return fail("limit depends on the call", n, fp32, 0, 0);
+    }
+    fld::launch_coarse_setup<double>(d, fld::Op<double>{}, nullptr, nullptr, nullptr, nullptr, false, nullptr);
+    if (g_lowered) return fail("limit depends on the call", n, 2, 0, 0);
+}
+if (g_limit.empty()) return fail("no limit recorded", 0, 0, 0, 0);
+"""
+
+
+def run_host(tmp_path, body, head='#include "walk4.cuh"\n'):
+    """Compiles body into a program with the library's code and runs it."""
     src = tmp_path / "plan.cu"
-    src.write_text('#include <cstdio>\n#include "walk4.cuh"\n'
+    src.write_text("#include <cstdio>\n" + head +
                    "static int fail(const char* what, int a, int b, int c, int d) {\n"
                    '    printf("%s: %d %d %d %d\\n", what, a, b, c, d);\n    return 1;\n}\n'
                    "int main() {\n" + body + "    return 0;\n}\n")
@@ -74,3 +105,9 @@ def test_prefetched_planes_lie_in_the_grid(tmp_path):
 
 def test_sweep_blocks_are_whole_warps(tmp_path):
     run_host(tmp_path, SHAPES)
+
+
+def test_shared_memory_limits_do_not_depend_on_the_call(tmp_path):
+    # the limit belongs to the function, so a smaller one set by one thread
+    # would refuse another thread's launch
+    run_host(tmp_path, LIMITS, RECORD)
