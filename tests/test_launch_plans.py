@@ -1,6 +1,6 @@
-"""Launch shapes and prefetch ranges that the library's headers compute on the
-host: a small program with the library's own inline functions is compiled and
-run here (no GPU)."""
+"""Launch shapes, limits, prefetch ranges and sums of the library's sources on
+the host: a small program with the library's own inline functions is compiled
+and run here (no GPU)."""
 import os
 import subprocess
 
@@ -82,6 +82,31 @@ for (int n : {64, 102, 125, 128, 130, 150, 160, 161, 300, 609, 693, 702, 760, 76
 if (g_limit.empty()) return fail("no limit recorded", 0, 0, 0, 0);
 """
 
+# The sum of 1024 threads' compensated pairs in the order of the one-CTA solve's
+# block sum: exact up to the two roundings of value(), as FP64 additions are
+# to a few (long double has 64 bits and more).
+SUMS = r"""
+unsigned long long x = 88172645463325252ull;
+auto uniform = [&]() {
+    x ^= x << 13; x ^= x >> 7; x ^= x << 17;
+    return (double)(x >> 11) * (1.0 / 9007199254740992.0);
+};
+for (int trial = 0; trial < 400; trial++) {
+    fld::DotSum v[1024];
+    long double exact = 0.0L;
+    for (auto& t : v) {
+        const float hi = (float)(uniform() * uniform() * uniform());
+        const float lo = (float)((uniform() - 0.5) * hi * 5.9e-8);
+        t = fld::DotSum{hi, lo, 0.0f};
+        exact += (long double)hi + (long double)lo;
+    }
+    for (int o = 1; o < 1024; o <<= 1)
+        for (int q = 0; q < 1024; q += 2 * o) v[q].merge(v[q + o].hi, v[q + o].lo, v[q + o].c);
+    const long double err = (long double)v[0].value() - exact;
+    if ((err < 0 ? -err : err) > 2.3e-16L * exact) return fail("block sum", trial, (int)(err / exact * 1e18L), 0, 0);
+}
+"""
+
 
 def run_host(tmp_path, body, head='#include "walk4.cuh"\n'):
     """Compiles body into a program with the library's code and runs it."""
@@ -111,3 +136,7 @@ def test_shared_memory_limits_do_not_depend_on_the_call(tmp_path):
     # the limit belongs to the function, so a smaller one set by one thread
     # would refuse another thread's launch
     run_host(tmp_path, LIMITS, RECORD)
+
+
+def test_block_sum_of_pairs_keeps_fp64_accuracy(tmp_path):
+    run_host(tmp_path, SUMS)
