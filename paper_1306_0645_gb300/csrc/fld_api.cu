@@ -2577,6 +2577,11 @@ fld_status fld_autotune(fld_ctx* c, int reps) {
         for (int k = 0; k < NTUNE && !st; k++) {
             if (k == TN_PMATVEC && l != 0) continue;
             if (k == TN_POST && !(c->p.fused_post && post4_ok(L.d))) continue;
+            if (k == TN_RESTRICT && comp && C.d.n <= RESTRICT_PAIR_CELLS) {
+                // launch_restrict_pair serves this level, with a shape of its own
+                L.tune[k] = Tune{};
+                continue;
+            }
             auto run = [&](const Tune& tn) {
                 switch (k) {
                 // the sweeps the V-cycle launches: bfloat16 coefficients where
@@ -2587,7 +2592,11 @@ fld_status fld_autotune(fld_ctx* c, int reps) {
                     else launch_smooth_zero4(L.d, L.A32, r, t, s, tn);
                     break;
                 case TN_RB:
-                    if (comp) launch_red8(L.d, L.Abf, r, t, z, nullptr, s, tn);
+                    if (comp) {
+                        // one record shapes both
+                        launch_black8(L.d, L.Abf, r, z, t + L.d.n / 2, s, tn);
+                        launch_red8(L.d, L.Abf, r, t + L.d.n / 2, z, nullptr, s, tn);
+                    }
                     else if (L.Abf.wx) launch_rb_colour4(L.d, L.Abf, r, t, 0, s, tn);
                     else launch_rb_colour4(L.d, L.A32, r, t, 0, s, tn);
                     break;
