@@ -6,6 +6,8 @@ shared library.  No CMake, no torch extension machinery.
 from __future__ import annotations
 
 import concurrent.futures as cf
+import functools
+import hashlib
 import os
 import shutil
 import subprocess
@@ -31,6 +33,17 @@ def nvcc() -> str:
 def _deps():
     files = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(INCLUDE, "fld.h")]
     return max(os.path.getmtime(f) for f in files)
+
+
+@functools.lru_cache(maxsize=None)
+def source_digest() -> str:
+    """Short digest of the library's sources: names one version of its kernels
+    (for files that hold what was measured with them)."""
+    h = hashlib.sha256()
+    for path in [os.path.join(CSRC, f) for f in sorted(os.listdir(CSRC))] + [os.path.join(INCLUDE, "fld.h")]:
+        with open(path, "rb") as f:
+            h.update(os.path.basename(path).encode() + b"\0" + f.read())
+    return h.hexdigest()[:12]
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

@@ -474,12 +474,17 @@ def fld_set_tuning(ctx: Context, table: Sequence[int]):
 
 def autotune(ctx: Context, cache_path: Optional[str] = None, reps: int = 3) -> List[int]:
     """Tune the context's FP32 launch shapes, or load them from a JSON cache
-    keyed by grid, boundaries, precision and GPU name; returns the table."""
+    keyed by what was tuned (grid, boundaries, precision, the options that choose
+    the sweeps, GPU name) and the version of the library's kernels, so shapes
+    measured with other kernels are never used; returns the table."""
     import json
     import torch
-    g = ctx._g
-    key = "%dx%dx%d_bc%d%d%d_p%d_%s" % (g.nx, g.ny, g.nz, g.bc[0], g.bc[1], g.bc[2], ctx.params.precision,
-                                         torch.cuda.get_device_name().replace(" ", "_"))
+    g, p = ctx._g, ctx.params
+    sweeps = (p.smoother, p.pre, p.post, p.paper_order, p.fused_post, p.precond_bf16, p.tail_cells)
+    key = "%dx%dx%d_bc%d%d%d_p%d_s%s_%s_%s" % (g.nx, g.ny, g.nz, g.bc[0], g.bc[1], g.bc[2], p.precision,
+                                               "-".join(map(str, sweeps)),
+                                               torch.cuda.get_device_name().replace(" ", "_"),
+                                               _build.source_digest())
     if cache_path is None:
         cache_path = os.environ.get("FLD_TUNE_CACHE",
                                     os.path.join(os.path.expanduser("~"), ".cache", "fld_gb300_tuning.json"))
