@@ -517,6 +517,29 @@ bool compressed_sweeps(const fld_ctx* c, int l) {
     return c->p.post == 1 && !c->p.paper_order && c->L[l].Abf.wx && fine8_ok(c->L[l].d);
 }
 
+// The tail from level l down: its levels and how they run; fits: whether the
+// plan does (always, for coarsest grids of at most COARSE_CAP_MAX cells).
+template <class T>
+TailArgs<T> tail_args(fld_ctx* c, int l, bool* fits) {
+    TailArgs<T> ta{};
+    ta.nlev = c->nl - l;
+    ta.pre = c->p.pre;
+    ta.post = c->p.post;
+    ta.paper_order = c->p.paper_order;
+    ta.ainv = c->ainv;
+    for (int q = 0; q < ta.nlev; q++) {
+        Level& Q = c->L[l + q];
+        TailLevel<T>& t = ta.L[q];
+        t.d = Q.d;
+        t.A = op_of<T>(Q);
+        t.r = (T*)Q.r;
+        t.z = (T*)Q.z;
+        t.t = (T*)Q.t;
+    }
+    *fits = plan_tail<T>(ta, c->tail_cluster, false);
+    return ta;
+}
+
 // z = B r on level l (zero initial guess).  If dot is given and the last
 // post-smoothing sweep of this level can carry it, <r, z> goes there (with
 // reduction *dot) and *dot_done is set.
@@ -533,26 +556,15 @@ void vcycle(fld_ctx* c, int l, const T* r, T* z, const RedArgs* dot = nullptr, b
         return;
     }
     if (l == c->tail_from) {
-        // this level and all coarser ones in one cluster launch
-        TailArgs<T> ta{};
-        ta.nlev = c->nl - l;
-        ta.pre = c->p.pre;
-        ta.post = c->p.post;
-        ta.paper_order = c->p.paper_order;
-        ta.ainv = c->ainv;
+        // this level and all coarser ones in one cluster launch (fld_create
+        // has checked that they fit)
+        bool fits = false;
+        TailArgs<T> ta = tail_args<T>(c, l, &fits);
+        ta.L[0].r = const_cast<T*>(r);
+        ta.L[0].z = z;
+        // smoothing, residual, transfers: about 30 words per cell
         double bytes = 0.0;
-        for (int q = 0; q < ta.nlev; q++) {
-            Level& Q = c->L[l + q];
-            TailLevel<T>& t = ta.L[q];
-            t.d = Q.d;
-            t.A = op_of<T>(Q);
-            t.r = q == 0 ? const_cast<T*>(r) : (T*)Q.r;
-            t.z = q == 0 ? z : (T*)Q.z;
-            t.t = (T*)Q.t;
-            // smoothing, residual, transfers: about 30 words per cell
-            bytes += 30.0 * (double)Q.d.n * ts;
-        }
-        plan_tail<T>(ta, c->tail_cluster, false);
+        for (int q = 0; q < ta.nlev; q++) bytes += 30.0 * (double)ta.L[q].d.n * ts;
         KScope k(c, K_VTAIL, bytes);
         launch_vtail<T>(ta, c->tail_cluster, s);
         return;
@@ -2132,7 +2144,12 @@ fld_status fld_create(fld_ctx** out, const fld_grid* g, const fld_params* p, voi
         int l0 = 0;
         while (l0 < c->nl - 1 && c->L[l0].d.n > cells) l0++;
         c->tail_cluster = c->mixed ? vtail_cluster<float>() : vtail_cluster<double>();
-        if (l0 < c->nl - 1 && c->nl - l0 <= TAIL_MAX_LEVELS && c->tail_cluster > 0) c->tail_from = l0;
+        if (l0 < c->nl - 1 && c->nl - l0 <= TAIL_MAX_LEVELS && c->tail_cluster > 0) {
+            bool fits = false;
+            if (c->mixed) tail_args<float>(c, l0, &fits);
+            else tail_args<double>(c, l0, &fits);
+            if (fits) c->tail_from = l0;
+        }
     }
     // persistent inner solves: the V-cycle over every level with the fine
     // level's CG vectors, written once to the context's device descriptor
@@ -2156,17 +2173,16 @@ fld_status fld_create(fld_ctx** out, const fld_grid* g, const fld_params* p, voi
         }
         ta.ainv = c->ainv;   // filled by every assembly
         R.cta = plan_tail<float>(ta, PS_CLUSTER, true) ? 1 : 0;
-        if (!R.cta) plan_tail<float>(ta, PS_CLUSTER, false);
+        c->ps = R.cta || plan_tail<float>(ta, PS_CLUSTER, false);
         R.x = (float*)c->cg[5];
         R.p = (float*)c->cg[2];
         R.q = (float*)c->cg[4];
         R.sc = c->sc;
-        if (cudaMemcpy(c->ps_req, &R, sizeof(R), cudaMemcpyHostToDevice) != cudaSuccess) {
+        if (c->ps && cudaMemcpy(c->ps_req, &R, sizeof(R), cudaMemcpyHostToDevice) != cudaSuccess) {
             cudaGetLastError();
             free_ctx(c);
             return set_err(FLD_ECUDA, "copy of the persistent-solve descriptor failed");
         }
-        c->ps = true;
     }
     {
         long long blocks = 0;

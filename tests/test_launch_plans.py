@@ -107,6 +107,48 @@ for (int trial = 0; trial < 400; trial++) {
 }
 """
 
+# Every tail that fld_create accepts (a coarsest grid of at most 4096 cells) has
+# a plan within its shared memory; a coarsest grid beyond that has none and is
+# reported, not launched.
+TAILS = r"""
+auto plan = [&](auto zero, const int (&c)[3], int nlev, int cluster, int sweeps, bool solve, int* bytes) {
+    fld::TailArgs<decltype(zero)> a{};
+    a.nlev = nlev;
+    a.pre = sweeps < 2 ? 1 : sweeps - 2;
+    a.post = sweeps < 2 ? 1 : 2;
+    a.paper_order = sweeps == 1;
+    for (int l = 0; l < nlev; l++) {
+        fld::Dims& d = a.L[l].d;
+        const int f = 1 << (nlev - 1 - l);
+        d.nx = c[0] * f; d.ny = c[1] * f; d.nz = c[2] * f;
+        d.n = (long long)d.nx * d.ny * d.nz;
+    }
+    const bool ok = fld::plan_tail(a, cluster, solve);
+    *bytes = a.smem_bytes;
+    return ok;
+};
+const int e[] = {1, 2, 3, 4, 5, 7, 8, 9, 15, 16, 17, 31, 32, 45, 64, 100, 128, 255, 512, 1000, 1024, 4096};
+int bytes = 0;
+for (int x : e)
+    for (int y : e)
+        for (int z : e) {
+            const int c[3] = {x, y, z};
+            if ((long long)x * y * z > 4096) continue;
+            for (int nlev = 2; nlev <= 5 && ((long long)x * y * z << 3 * (nlev - 1)) <= (1 << 24); nlev++)
+                for (int cluster : {8, 16})
+                    for (int sweeps = 0; sweeps < 4; sweeps++) {
+                        if (!plan(0.0f, c, nlev, cluster, sweeps, false, &bytes) || bytes > (int)fld::TAIL_SMEM_MAX)
+                            return fail("FP32 tail", x, y, z, nlev);
+                        if (!plan(0.0, c, nlev, cluster, sweeps, false, &bytes) || bytes > (int)fld::TAIL_SMEM_MAX)
+                            return fail("FP64 tail", x, y, z, nlev);
+                        if (plan(0.0f, c, nlev, cluster, sweeps, true, &bytes) && bytes > (int)fld::PS_SMEM_MAX)
+                            return fail("one-CTA solve", x, y, z, nlev);
+                    }
+        }
+const int big[3] = {32, 32, 32};
+if (plan(0.0, big, 2, 16, 0, false, &bytes)) return fail("a coarsest grid that does not fit", 32, 32, 32, bytes);
+"""
+
 
 def run_host(tmp_path, body, head='#include "walk4.cuh"\n'):
     """Compiles body into a program with the library's code and runs it."""
@@ -140,3 +182,7 @@ def test_shared_memory_limits_do_not_depend_on_the_call(tmp_path):
 
 def test_block_sum_of_pairs_keeps_fp64_accuracy(tmp_path):
     run_host(tmp_path, SUMS)
+
+
+def test_every_accepted_tail_has_a_plan(tmp_path):
+    run_host(tmp_path, TAILS, '#include "k_tail.cu"\n')
