@@ -553,8 +553,10 @@ void launch_coarse_setup(const Dims& d, Op<T> A, double* dense, double* ainv, do
             other = t;
         }
     }
-    // columns per CTA: one wave of CTAs up to 5 columns each, beyond that 4
-    // while their x and r fit 96 KB (k_coarse_refine)
+    // columns per CTA: one wave of CTAs up to 5 columns each (693 cells: 162 us
+    // with 5 columns, 276 with 4 in two uneven waves of 256 threads), beyond
+    // that 4 while their x and r fit 96 KB (k_coarse_refine).  Six to eight
+    // columns, one wave up to 1216 cells, were not measured.
     if (n <= 152) refine_go<T, 1>(d, A, M, ainv, flag, s);
     else if (n <= 2 * 152) refine_go<T, 2>(d, A, M, ainv, flag, s);
     else if (n <= 3 * 152) refine_go<T, 3>(d, A, M, ainv, flag, s);

@@ -2,7 +2,7 @@
 // per thread, one red and one black.
 //
 // GB300 has two FP64 lanes per SM and clock, so these kernels are bound by FP64
-// instructions first (1.05 M pairs at 128^3: 3.6 us per FP64 instruction and
+// instructions first (1.05 M pairs at 128^3: 1.8 us per FP64 instruction and
 // pair), then by L2 and DRAM.  The scalar kernels of k_mg.cu and k_cg.cu issue
 // an instruction for a whole warp where a colour needs half its lanes, form a
 // red neighbour's r / diag again for each of its six black neighbours, r - A z
